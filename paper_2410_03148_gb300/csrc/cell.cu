@@ -232,6 +232,15 @@ struct Krylov {
 
 }  // namespace
 
+// Modal matrices of the operators on one grid (mm2 materials, modal.cuh).
+template <typename T>
+struct ModalSet {
+  cell::ModalMat<T, 4, 4> full;
+  cell::ModalMat<T, 3, 3> uu;
+  cell::ModalMat<T, 1, 3> pu;
+  cell::ModalSch<T> ss;
+};
+
 struct cell_handle {
   cell_desc d{};
   int dev = 0;             // CUDA device current at set-up
@@ -242,6 +251,10 @@ struct cell_handle {
   double Cn[36], en[18], kn[9];
   double h[3];
   double K0[1024], S0[64], Z[288], F[288], H0e[81];
+  bool modal = false;            // mm2 material: operators in modal form
+  ModalSet<float> m32;
+  ModalSet<double> m64;
+  cell::ModalMat<cell::DF, 4, 4> mdf;
   Arena arena;
   float* rho32 = nullptr;
   double* rho64 = nullptr;
@@ -320,6 +333,37 @@ int tune_tiles(cell_handle* h);
 template <typename T, int NC> void tune_stencils(cell_handle* h, BlockMG<T>& mg);
 void tile_stats(const cell_handle* h, cell_stats& S);
 template <> Krylov<double>& kry<double>(cell_handle* h) { return h->kd; }
+
+template <typename T> const ModalSet<T>& modal_of(const cell_handle* h);
+template <> const ModalSet<float>& modal_of<float>(const cell_handle* h) { return h->m32; }
+template <> const ModalSet<double>& modal_of<double>(const cell_handle* h) { return h->m64; }
+
+// Blocks of one, two and three differences of rows o0 .. o0 + NO - 1 and
+// columns 0 .. NI - 1 of a modal matrix over nc components.
+template <int NO, int NI, typename V, typename F>
+void fill_modal(const double* Km, int nc, int o0, cell::ModalMat<V, NO, NI>& M, F&& conv) {
+  const int R = 8 * nc;
+  auto at = [&](int m, int c, int n, int d) { return conv(Km[(m * nc + o0 + c) * R + n * nc + d]); };
+  for (int c = 0; c < NO; ++c)
+    for (int d = 0; d < NI; ++d) {
+      for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) {
+          const int k = (i * NO + c) * 3 * NI + j * NI + d;
+          M.c[k] = at(1 << i, c, 1 << j, d);
+          M.q[k] = at(7 ^ (1 << i), c, 7 ^ (1 << j), d);
+        }
+      M.t[c * NI + d] = at(7, c, 7, d);
+    }
+}
+
+template <typename T>
+void fill_modal_set(const double* Km, const double* Sm, ModalSet<T>& M) {
+  auto conv = [](double v) { return (T)v; };
+  fill_modal<4, 4, T>(Km, 4, 0, M.full, conv);
+  fill_modal<3, 3, T>(Km, 4, 0, M.uu, conv);
+  fill_modal<1, 3, T>(Km, 4, 3, M.pu, conv);
+  for (int m = 0; m < 8; ++m) M.ss.s[m] = (T)Sm[m * 8 + m];
+}
 
 template <typename T> const T* rho_of(cell_handle* h);
 template <> const float* rho_of<float>(cell_handle* h) { return h->rho32; }
@@ -640,6 +684,27 @@ void block_solve(cell_handle* h, BlockMG<T>& mg, int cycles, const T* b, i64 bs,
   }
 }
 
+// Arguments of a modal operator on the finest grid.
+template <typename T>
+cell::ModalArgs<T> modal_args(cell_handle* h, const T* x, i64 xs, T* y, i64 ys, int nrhs, const int* mask) {
+  cell::ModalArgs<T> m{};
+  m.x = x; m.xs = xs; m.y = y; m.ys = ys;
+  m.rho = rho_of<T>(h); m.nx = h->nx; m.ny = h->ny; m.nz = h->nz;
+  m.nrhs = nrhs; m.active = mask;
+  return m;
+}
+
+// FP64-grade residual r = b - Ahat x of the split iterate (x = xh + xl)
+void residual_df(cell_handle* h, const double* b, double* r, int nrhs) {
+  const i64 len = 4 * h->nn;
+  if (h->modal)
+    cell::modal_resid_df(h->xh, h->xl, len, b, len, r, len, h->rho32, h->rho_l, h->mdf, h->nx, h->ny, h->nz, nrhs,
+                         h->st);
+  else
+    cell::resid_df(h->xh, h->xl, len, b, len, r, len, h->rho32, h->rho_l, h->DF, h->nx, h->ny, h->nz, nrhs, nullptr,
+                   h->st);
+}
+
 // z = P_SCP^-1 v (§2.5.3): z_u ~ A^-1 v_u, z_phi ~ Sbar^-1 (v_phi + B z_u).
 template <typename T>
 void precond(cell_handle* h, const T* v, T* z, const int* mask) {
@@ -657,25 +722,41 @@ void precond(cell_handle* h, const T* v, T* z, const int* mask) {
   a.active = mask;
   a.cslot1 = h->cslot1;
   const int ip = h->prof.begin(h->st, CELL_PROF_COUPLING);
-  cell::apply_pu<T>(a, K.K0, 9, h->st);
+  if (h->modal) {
+    cell::ModalArgs<T> m = modal_args<T>(h, z, len, K.tphi, nn, 9, mask);
+    m.b = v + 3 * nn; m.bs = len;
+    cell::modal_pu<T>(m, modal_of<T>(h).pu, cell::MM_ADD, h->st);
+  } else {
+    cell::apply_pu<T>(a, K.K0, 9, h->st);
+  }
   h->prof.end(CELL_PROF_COUPLING, ip, h->st);
   block_solve<T, 1>(h, K.mgp, h->d.opt.vcycles_phi, K.tphi, nn, z + 3 * nn, len, K.rp, K.ep, mask);
 }
 
+// y = Ahat x, or y = b - Ahat x with b set.
 template <typename T>
-void apply_full_T(cell_handle* h, const T* x, i64 xs, T* y, i64 ys, const T* b, i64 bs, T alpha,
-                  T beta, const int* mask, int nrhs) {
+void apply_full_T(cell_handle* h, const T* x, i64 xs, T* y, i64 ys, const T* b, i64 bs, const int* mask, int nrhs) {
   cell::ApplyArgs<T> a{};
-  a.x = x; a.xs = xs; a.y = y; a.ys = ys; a.b = b; a.bs = bs; a.alpha = alpha; a.beta = beta;
+  a.x = x; a.xs = xs; a.y = y; a.ys = ys; a.b = b; a.bs = bs; a.alpha = b ? T(-1) : T(1); a.beta = T(1);
   a.rho = rho_of<T>(h); a.nx = h->nx; a.ny = h->ny; a.nz = h->nz; a.active = mask;
   a.cslot1 = h->cslot1;
   const int pcls = sizeof(T) == 4 ? CELL_PROF_FULL32 : CELL_PROF_FULL64;
   const int ip = h->prof.begin(h->st, pcls);
+  bool done = false;
   if constexpr (sizeof(T) == 4) {
-    if (h->tc_ok && h->d.opt.tensor_cores >= 2) cell::apply_tc_full(a, h->tct, nrhs, h->tc_err, h->st);
-    else cell::apply_full<T>(a, h->kf.K0, cell::AM_LINEAR, nrhs, h->st);
-  } else {
-    cell::apply_full<T>(a, h->kd.K0, cell::AM_LINEAR, nrhs, h->st);
+    if (h->tc_ok && h->d.opt.tensor_cores >= 2) {
+      cell::apply_tc_full(a, h->tct, nrhs, h->tc_err, h->st);
+      done = true;
+    }
+  }
+  if (!done && h->modal) {
+    cell::ModalArgs<T> m = modal_args<T>(h, x, xs, y, ys, nrhs, mask);
+    m.b = b; m.bs = bs;
+    cell::modal_full<T>(m, modal_of<T>(h).full, b ? cell::MM_RESID : cell::MM_APPLY, h->st);
+  } else if (!done) {
+    cell::FixedMat<T, 4> M;
+    for (int i = 0; i < 1024; ++i) M.k[i] = (T)h->K0[i];
+    cell::apply_full<T>(a, M, cell::AM_LINEAR, nrhs, h->st);
   }
   h->prof.end(pcls, ip, h->st);
 }
@@ -735,7 +816,7 @@ void iteration(cell_handle* h, int j) {
   T* w = K.V + (i64)(j + 1) * vstride;
   T* zj = K.Z + (i64)j * vstride;
   precond<T>(h, vj, zj, h->active);
-  apply_full_T<T>(h, zj, len, w, len, nullptr, 0, T(1), T(0), h->active, 9);
+  apply_full_T<T>(h, zj, len, w, len, nullptr, 0, h->active, 9);
   // Classical Gram-Schmidt with selective reorthogonalisation: one pass of
   // dots (w is V_{j+1}, so the same pass also gives |w|^2); one pass that
   // updates w and, from the same basis reads, forms the second pass's dots
@@ -944,6 +1025,18 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
     // dielectric block C_e itself (K0 = [[A, B^T], [B, -C]]), no coupling
     for (int a = 0; a < 8; ++a)
       for (int b = 0; b < 8; ++b) h->S0[a * 8 + b] = -h->K0[(4 * a + 3) * 32 + 4 * b + 3];
+  }
+  h->modal = cellhost::is_mm2(d->C, d->e, d->kappa);
+  if (h->modal) {
+    double Km[1024], Sm[64];
+    cellhost::modal_matrix(h->K0, 4, Km);
+    cellhost::modal_matrix(h->S0, 1, Sm);
+    fill_modal_set(Km, Sm, h->m32);
+    fill_modal_set(Km, Sm, h->m64);
+    fill_modal<4, 4, cell::DF>(Km, 4, 0, h->mdf, [](double v) {
+      const float hi = (float)v;
+      return cell::DF{hi, (float)(v - (double)hi)};
+    });
   }
   cellhost::affine_loads(h->h, h->Z);
   for (int a = 0; a < 32; ++a)
@@ -1212,10 +1305,9 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
         cell::axpy_f64<T>(h->x64, len, K.u, len, len, h->ones, 9, h->ranmask, s);
       cell::accum_iters(h->iters_d, h->kcount, h->ranmask, h->ctl_d, s);
       if constexpr (sizeof(T) == 4)
-        cell::resid_df(h->xh, h->xl, len, h->b64, len, h->r64, len, h->rho32, h->rho_l, h->DF, h->nx, h->ny,
-                       h->nz, 9, nullptr, s);
+        residual_df(h, h->b64, h->r64, 9);
       else
-        apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, -1.0, 1.0, nullptr, 9);
+        apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, nullptr, 9);
       cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
       cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->red, 0, 9, nullptr, s);
       cell::refine_ctl(h->bn2d, h->red, h->bfloor_d, P, h->want, h->tolabs, h->relres_d, h->iters_d, h->ctl_d, wh, s);
@@ -1375,11 +1467,10 @@ int solve_impl(cell_handle* h, cell_stats* st) {
     h->prof.cur_units = 9;
     if constexpr (sizeof(T) == 4) {
       const int ip = h->prof.begin(s, CELL_PROF_FULL64);
-      cell::resid_df(h->xh, h->xl, len, h->b64, len, h->r64, len, h->rho32, h->rho_l, h->DF,
-                     h->nx, h->ny, h->nz, 9, nullptr, s);
+      residual_df(h, h->b64, h->r64, 9);
       h->prof.end(CELL_PROF_FULL64, ip, s);
     } else {
-      apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, -1.0, 1.0, nullptr, 9);
+      apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, nullptr, 9);
     }
   }
   // null-space projection (mean displacement and potential per load)
@@ -2010,21 +2101,30 @@ int cell_get_solution(cell_handle* h, double* out) {
 int cell_apply(cell_handle* h, const void* x, void* y, int nrhs, int dtype) {
   if (!h || !x || !y || nrhs < 1 || nrhs > 65535) return CELL_EINVAL;
   const i64 len = 4 * h->nn;
-  if (dtype == CELL_F32) {
-    cell::ApplyArgs<float> a{};
-    a.x = static_cast<const float*>(x); a.xs = len; a.y = static_cast<float*>(y); a.ys = len;
-    a.alpha = 1.f; a.rho = h->rho32; a.nx = h->nx; a.ny = h->ny; a.nz = h->nz;
-    a.cslot1 = h->cslot1;   // the kernels the solver runs
-    cell::FixedMat<float, 4> M;
-    for (int i = 0; i < 1024; ++i) M.k[i] = (float)h->K0[i];
-    cell::apply_full<float>(a, M, cell::AM_LINEAR, nrhs, h->st);
-  } else if (dtype == CELL_F64) {
-    cell::ApplyArgs<double> a{};
-    a.x = static_cast<const double*>(x); a.xs = len; a.y = static_cast<double*>(y); a.ys = len;
-    a.alpha = 1.0; a.rho = h->rho64; a.nx = h->nx; a.ny = h->ny; a.nz = h->nz;
-    cell::FixedMat<double, 4> M;
-    std::memcpy(M.k, h->K0, sizeof(M.k));
-    cell::apply_full<double>(a, M, cell::AM_LINEAR, nrhs, h->st);
+  if (dtype == CELL_F32 || dtype == CELL_F64) {
+    if (h->modal) {
+      if (dtype == CELL_F32)
+        cell::modal_full<float>(modal_args<float>(h, static_cast<const float*>(x), len, static_cast<float*>(y), len,
+                                                  nrhs, nullptr), h->m32.full, cell::MM_APPLY, h->st);
+      else
+        cell::modal_full<double>(modal_args<double>(h, static_cast<const double*>(x), len, static_cast<double*>(y),
+                                                    len, nrhs, nullptr), h->m64.full, cell::MM_APPLY, h->st);
+    } else if (dtype == CELL_F32) {
+      cell::ApplyArgs<float> a{};
+      a.x = static_cast<const float*>(x); a.xs = len; a.y = static_cast<float*>(y); a.ys = len;
+      a.alpha = 1.f; a.rho = h->rho32; a.nx = h->nx; a.ny = h->ny; a.nz = h->nz;
+      a.cslot1 = h->cslot1;   // the kernels the solver runs
+      cell::FixedMat<float, 4> M;
+      for (int i = 0; i < 1024; ++i) M.k[i] = (float)h->K0[i];
+      cell::apply_full<float>(a, M, cell::AM_LINEAR, nrhs, h->st);
+    } else {
+      cell::ApplyArgs<double> a{};
+      a.x = static_cast<const double*>(x); a.xs = len; a.y = static_cast<double*>(y); a.ys = len;
+      a.alpha = 1.0; a.rho = h->rho64; a.nx = h->nx; a.ny = h->ny; a.nz = h->nz;
+      cell::FixedMat<double, 4> M;
+      std::memcpy(M.k, h->K0, sizeof(M.k));
+      cell::apply_full<double>(a, M, cell::AM_LINEAR, nrhs, h->st);
+    }
   } else if (dtype == CELL_F32_TC) {
     if (!h->tc_ok) return CELL_EINVAL;
     cell::ApplyArgs<float> a{};
@@ -2034,8 +2134,7 @@ int cell_apply(cell_handle* h, const void* x, void* y, int nrhs, int dtype) {
   } else if (dtype == CELL_F64_DF) {
     if (nrhs > 9) return CELL_EINVAL;
     cell::split_f64(static_cast<const double*>(x), h->xh, h->xl, (i64)nrhs * len, h->st);
-    cell::resid_df(h->xh, h->xl, len, nullptr, 0, static_cast<double*>(y), len, h->rho32, h->rho_l,
-                   h->DF, h->nx, h->ny, h->nz, nrhs, nullptr, h->st);
+    residual_df(h, nullptr, static_cast<double*>(y), nrhs);
   } else {
     return CELL_EINVAL;
   }
@@ -2069,7 +2168,19 @@ int cell_apply_block(cell_handle* h, int block, const void* x, void* y, int nrhs
   if (block != CELL_BLOCK_A && block != CELL_BLOCK_SBAR) return CELL_EINVAL;
   const int nc = block == CELL_BLOCK_A ? 3 : 1;
   const i64 len = nc * h->nn;
-  if (dtype == CELL_F32 || dtype == CELL_F32_TC) {
+  if (h->modal && (dtype == CELL_F32 || dtype == CELL_F64)) {
+    if (dtype == CELL_F32) {
+      const cell::ModalArgs<float> m = modal_args<float>(h, static_cast<const float*>(x), len, static_cast<float*>(y),
+                                                         len, nrhs, nullptr);
+      if (nc == 3) cell::modal_uu<float>(m, h->m32.uu, cell::MM_APPLY, h->st);
+      else cell::modal_ss<float>(m, h->m32.ss, cell::MM_APPLY, h->st);
+    } else {
+      const cell::ModalArgs<double> m = modal_args<double>(h, static_cast<const double*>(x), len,
+                                                           static_cast<double*>(y), len, nrhs, nullptr);
+      if (nc == 3) cell::modal_uu<double>(m, h->m64.uu, cell::MM_APPLY, h->st);
+      else cell::modal_ss<double>(m, h->m64.ss, cell::MM_APPLY, h->st);
+    }
+  } else if (dtype == CELL_F32 || dtype == CELL_F32_TC) {
     cell::ApplyArgs<float> a{};
     a.x = static_cast<const float*>(x); a.xs = len; a.y = static_cast<float*>(y); a.ys = len;
     a.alpha = 1.f; a.rho = h->rho32; a.nx = h->nx; a.ny = h->ny; a.nz = h->nz;

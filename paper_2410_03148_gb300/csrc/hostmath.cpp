@@ -261,6 +261,43 @@ int spd_inverse(double* A, int n) {
   return 0;
 }
 
+bool is_mm2(const double C[36], const double e[18], const double kap[9]) {
+  for (int i = 0; i < 6; ++i)
+    for (int j = 0; j < 6; ++j)
+      if (i != j && !(i < 3 && j < 3) && C[i * 6 + j] != 0.0) return false;
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 6; ++j) {
+      const bool used = (i == 2 && j < 3) || (i == 0 && j == 4) || (i == 1 && j == 3);
+      if (!used && e[i * 6 + j] != 0.0) return false;
+    }
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j)
+      if (i != j && kap[i * 3 + j] != 0.0) return false;
+  return true;
+}
+
+void modal_matrix(const double* K, int nc, double* Km) {
+  const int R = 8 * nc;
+  // 64 terms cancel: transformed in extended precision, so that the entries
+  // are the ones of K to its last digit
+  std::vector<long double> M(K, K + R * R);
+  for (int side = 0; side < 2; ++side)
+    for (int bit = 1; bit < 8; bit <<= 1)
+      for (int a = 0; a < 8; ++a) {
+        if (a & bit) continue;
+        for (int c = 0; c < nc; ++c)
+          for (int k = 0; k < R; ++k) {
+            const int lo = a * nc + c, hi = (a | bit) * nc + c;
+            long double& u = side ? M[k * R + lo] : M[lo * R + k];
+            long double& v = side ? M[k * R + hi] : M[hi * R + k];
+            const long double s = v + u, d = v - u;   // sum at the clear bit, difference at the set one
+            u = s;
+            v = d;
+          }
+      }
+  for (int i = 0; i < R * R; ++i) Km[i] = (double)(M[i] / 64.0L);
+}
+
 double child_weight(int c, int a, int B) {
   double w = 1.0;
   for (int d = 0; d < 3; ++d) {

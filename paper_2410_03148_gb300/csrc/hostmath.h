@@ -22,6 +22,16 @@ void affine_loads(const double h[3], double Z[32 * 9]);
 // 8x8 S0 = C_e + B_e (A_e + shift I)^-1 B_e^T from the element matrix (§2.5.3).
 int local_schur(const double K[1024], double shift, double S[64]);
 
+// Material with the mm2 mirror planes of the grid axes: no normal-shear or
+// shear-shear coupling in C, e with e31, e32, e33, e15, e24 only, diagonal
+// kappa (every other entry exactly zero).
+bool is_mm2(const double C[36], const double e[18], const double kap[9]);
+
+// Modal form of an element matrix over 8 nodes with nc components (local dof
+// nc * node + c): Km = H K H^T / 64 with H the sums and differences along the
+// axes, Km[(m * nc + c) * 8 nc + n * nc + d], so that K = H^T Km H.
+void modal_matrix(const double* K, int nc, double* Km);
+
 // Upper bound of lambda_max(diag(M)^-1 M) for a symmetric n x n matrix.
 double jacobi_lmax(const double* M, int n);
 

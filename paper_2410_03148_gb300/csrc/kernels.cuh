@@ -96,6 +96,60 @@ struct ApplyArgs {
   int nrhs;                // number of loads of the launch (set by the launchers)
 };
 
+// ---- modal element operators (modal.cuh, modal_f32.cu, modal_f64.cu) -----------
+enum ModalKind { MK_FULL = 0, MK_UU = 1, MK_PU = 2, MK_SS = 3 };   // Ahat, A, B, Sbar
+enum ModalMode {
+  MM_APPLY = 0,   // y = A x
+  MM_ADD = 1,     // y = b + A x
+  MM_RESID = 2,   // y = b - A x
+  // Chebyshev-Jacobi steps on A x = b in three-term form, D = diag(A):
+  //   x_{k+1} = x_k + c1 (x_k - x_{k-1}) + c2 D^-1 (b - A x_k)
+  MM_STEP = 3,    // y = x_{k+1}, x_{k-1} = xp (y may be xp)
+  MM_STEP0 = 4,   // the same with x_{k-1} = c0 D^-1 b
+  MM_PRE = 5,     // the same with x_k = c0 D^-1 b (not stored) and x_{k-1} = 0
+  MM_POST = 6     // y = x + c2 D^-1 (b - A x)
+};
+// Modal element matrix K^ (modal.cuh), blocks of one (c), two (q) and three
+// (t) differences: c[(i NO + c) 3 NI + j NI + d] couples output component c of
+// the mode "difference along i" with input component d of "difference along
+// j"; q likewise for the modes "difference along all axes but i".
+template <typename T, int NO, int NI>
+struct ModalMat {
+  T c[9 * NO * NI], q[9 * NO * NI], t[NO * NI];
+};
+template <typename T>
+struct ModalSch {   // diagonal of Sbar's modal matrix, modes 1..7
+  T s[8];
+};
+struct DF {         // unevaluated pair h + l
+  float h, l;
+};
+// One operator launch.  Vectors as in ApplyArgs: value(load q, comp c, node n)
+// = p[q * stride + c * nn + n].
+template <typename T>
+struct ModalArgs {
+  const T* x; i64 xs;      // gathered input (MM_PRE: unused)
+  T* y; i64 ys;            // output
+  const T* b; i64 bs;      // right-hand side (all modes but MM_APPLY)
+  const T* xp; i64 ps;     // MM_STEP: x_{k-1}
+  const T* dinv;           // inverse diagonal [NC][nn] (steps)
+  const T* rho;            // element scales
+  const T* c12;            // device (c1, c2) of the step
+  const T* c0;             // device c0 of the first step (MM_STEP0, MM_PRE)
+  int nx, ny, nz;
+  const int* active;       // per-load flag (nullptr = all)
+  int nrhs;
+  int rg;                  // loads per block, one after another (0 = 1)
+};
+template <typename T> void modal_full(const ModalArgs<T>& a, const ModalMat<T, 4, 4>& K, int mode, cudaStream_t s);
+template <typename T> void modal_pu(const ModalArgs<T>& a, const ModalMat<T, 1, 3>& K, int mode, cudaStream_t s);
+template <typename T> void modal_uu(const ModalArgs<T>& a, const ModalMat<T, 3, 3>& K, int mode, cudaStream_t s);
+template <typename T> void modal_ss(const ModalArgs<T>& a, const ModalSch<T>& K, int mode, cudaStream_t s);
+// FP64-grade r = b - Ahat x (r = Ahat x if b is null) in pairs of FP32, as resid_df
+void modal_resid_df(const float* xh, const float* xl, i64 xs, const double* b, i64 bs, double* r, i64 rs,
+                    const float* rho_h, const float* rho_l, const ModalMat<DF, 4, 4>& K, int nx, int ny, int nz,
+                    int nrhs, cudaStream_t s);
+
 // Constant-bank slots holding (K0, S0) in FP32 for the fixed-matrix kernels;
 // returns slot + 1, or 0 if none is free.  Release with cslot_release.
 int cslot_acquire(const float* K0f, const float* S0f);

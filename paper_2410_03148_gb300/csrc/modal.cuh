@@ -1,0 +1,378 @@
+// Element operators in their modal form (included by the modal_*.cu units).
+//
+// On a box element the 8 corner values of a component are replaced by their
+// sums and differences along the axes, u^_m with m = (x, y, z) bits, bit set =
+// difference (u(1) - u(0)), clear = sum.  In this basis the Q1 element matrix
+// K = H^T K^ H is sparse: it couples only modes of the same number of
+// differences (one: the constant strains; two: the linear ones; three), and
+// constants drop out.  For a material with the mm2 mirror planes (no
+// normal-shear coupling, e only e31 e32 e33 e15 e24, diagonal kappa: poled
+// ceramics on an aligned grid) it couples only dofs of equal parity under
+// the three mirrors as well: 82 products for the coupled operator against
+// 1024 of the corner form, 45 (of 576) for the elastic block, 7 (of 64) for
+// Sbar, 15 (of 192) for the coupling block.  The transforms are shared between
+// neighbours: per node and component 2 operations along x, 4 along y and 7
+// along z, and 19 back.  Other materials keep the corner form (apply.cu): with
+// all 304 products of the modal matrix the registers of a thread do not hold
+// the modes of an element.
+//
+// One warp owns a strip of RY node rows by 30 columns (lanes 1..30; lanes 0
+// and 31 are halo) and marches through z.  x neighbours are lane shuffles, y
+// neighbours the rows a thread holds, z neighbours registers carried from the
+// plane before: no shared memory, no barrier, no atomics, and every element
+// is evaluated once per strip (RY + 1 element rows for RY node rows).  The
+// columns of all strips form one sequence of nx + 2 positions per strip (both
+// periodic ends included), which warps cut into windows of 30 outputs, so any
+// nx keeps about 30/32 of the lanes busy.
+#pragma once
+
+#include "kernels.cuh"
+
+namespace cell {
+namespace modal {
+
+constexpr int kThreads = 128;
+constexpr int kWarps = kThreads / 32;
+constexpr int kOut = 30;   // output columns of a warp
+
+// Mirror parity of dof (component c, mode m): a displacement component and
+// its own axis' difference flip together; the potential flips with z.
+__host__ __device__ constexpr int parity(int c, int m) { return m ^ (c == 0 ? 1 : (c == 1 ? 2 : 4)); }
+__host__ __device__ constexpr bool couples(int c, int m, int c2, int m2) { return parity(c, m) == parity(c2, m2); }
+
+// ---- arithmetic -------------------------------------------------------------
+// Value types: float, double, and DF, an unevaluated pair h + l of floats with
+// error-free products and sums of the leading parts (about 2^-46).
+__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
+__device__ __forceinline__ float vsub(float a, float b) { return a - b; }
+__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ DF vadd(DF a, DF b) {
+  const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+  return {s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
+}
+__device__ __forceinline__ DF vsub(DF a, DF b) { return vadd(a, DF{-b.h, -b.l}); }
+__device__ __forceinline__ DF vmul(DF a, DF b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return {p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ DF vfma(DF a, DF b, DF c) { return vadd(c, vmul(a, b)); }
+
+__device__ __forceinline__ float vdown(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ double vdown(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ DF vdown(DF v) { return {vdown(v.h), vdown(v.l)}; }
+__device__ __forceinline__ float vup(float v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ double vup(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ DF vup(DF v) { return {vup(v.h), vup(v.l)}; }
+
+// Two values that differ in the x mode (sum, difference).  FP32 pairs use the
+// packed instructions (two results per issue slot); a - b is fma(b, -1, a),
+// the same rounding.
+template <typename V>
+struct Pair {
+  V s, d;
+};
+template <>
+struct Pair<float> {
+  float2 p;
+};
+template <typename V> __device__ __forceinline__ V sum_of(const Pair<V>& a) { return a.s; }
+template <typename V> __device__ __forceinline__ V dif_of(const Pair<V>& a) { return a.d; }
+__device__ __forceinline__ float sum_of(const Pair<float>& a) { return a.p.x; }
+__device__ __forceinline__ float dif_of(const Pair<float>& a) { return a.p.y; }
+template <typename V> __device__ __forceinline__ Pair<V> mk(V s, V d) { return {s, d}; }
+template <> __device__ __forceinline__ Pair<float> mk<float>(float s, float d) { return {make_float2(s, d)}; }
+template <typename V> __device__ __forceinline__ Pair<V> padd(const Pair<V>& a, const Pair<V>& b) {
+  return {vadd(a.s, b.s), vadd(a.d, b.d)};
+}
+template <typename V> __device__ __forceinline__ Pair<V> psub(const Pair<V>& a, const Pair<V>& b) {
+  return {vsub(a.s, b.s), vsub(a.d, b.d)};
+}
+template <typename V> __device__ __forceinline__ Pair<V> pmul(V k, const Pair<V>& a) {
+  return {vmul(k, a.s), vmul(k, a.d)};
+}
+__device__ __forceinline__ Pair<float> padd(const Pair<float>& a, const Pair<float>& b) {
+  return {__fadd2_rn(a.p, b.p)};
+}
+__device__ __forceinline__ Pair<float> psub(const Pair<float>& a, const Pair<float>& b) {
+  return {__ffma2_rn(b.p, make_float2(-1.f, -1.f), a.p)};
+}
+__device__ __forceinline__ Pair<float> pmul(float k, const Pair<float>& a) {
+  return {__fmul2_rn(make_float2(k, k), a.p)};
+}
+
+// ---- element contraction ------------------------------------------------------
+// f[c][m] = sum K^[(c,m)][(d,n)] u[d][n] within the classes of one, two and
+// three differences.  CO = component of the first output row.
+//
+// first input dof (j NI + d, from 0) that row (c, mode) of a class couples
+// with; mode of axis j: 1 << j, or 7 without it
+template <int NI>
+__host__ __device__ constexpr int first_of(int c, int m, bool two) {
+  for (int k = 0; k < 3 * NI; ++k)
+    if (couples(c, m, k % NI, two ? 7 ^ (1 << (k / NI)) : 1 << (k / NI))) return k;
+  return -1;
+}
+template <int NI>
+__host__ __device__ constexpr int first_of3(int c) {
+  for (int d = 0; d < NI; ++d)
+    if (couples(c, 7, d, 7)) return d;
+  return -1;
+}
+
+template <int NO, int NI, int CO, typename V>
+__device__ __forceinline__ void force(const ModalMat<V, NO, NI>& K, const V (&u)[NI][8], V (&f)[NO][8]) {
+#pragma unroll
+  for (int c = 0; c < NO; ++c) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int m1 = 1 << i, m2 = 7 ^ m1;
+      V f1 = V{}, f2 = V{};
+#pragma unroll
+      for (int k = 0; k < 3 * NI; ++k) {
+        const int j = k / NI, d = k % NI, n1 = 1 << j, n2 = 7 ^ n1, at = (i * NO + c) * 3 * NI + k;
+        if (couples(CO + c, m1, d, n1))
+          f1 = k == first_of<NI>(CO + c, m1, false) ? vmul(K.c[at], u[d][n1]) : vfma(K.c[at], u[d][n1], f1);
+        if (couples(CO + c, m2, d, n2))
+          f2 = k == first_of<NI>(CO + c, m2, true) ? vmul(K.q[at], u[d][n2]) : vfma(K.q[at], u[d][n2], f2);
+      }
+      f[c][m1] = f1;
+      f[c][m2] = f2;
+    }
+    V f3 = V{};
+#pragma unroll
+    for (int d = 0; d < NI; ++d)
+      if (couples(CO + c, 7, d, 7))
+        f3 = d == first_of3<NI>(CO + c) ? vmul(K.t[c * NI + d], u[d][7]) : vfma(K.t[c * NI + d], u[d][7], f3);
+    f[c][7] = f3;
+  }
+}
+// Sbar: the three mirrors leave every mode alone, S^ is diagonal.
+template <typename V>
+__device__ __forceinline__ void force_s(const ModalSch<V>& K, const V (&u)[1][8], V (&f)[1][8]) {
+#pragma unroll
+  for (int m = 1; m < 8; ++m) f[0][m] = vmul(K.s[m], u[0][m]);
+}
+
+template <int KIND>
+struct Shape;   // input and output components
+template <> struct Shape<MK_FULL> { static constexpr int NI = 4, NO = 4, CO = 0; };
+template <> struct Shape<MK_UU> { static constexpr int NI = 3, NO = 3, CO = 0; };
+template <> struct Shape<MK_PU> { static constexpr int NI = 3, NO = 1, CO = 3; };
+template <> struct Shape<MK_SS> { static constexpr int NI = 1, NO = 1, CO = 0; };
+
+template <int KIND, typename V>
+struct MatOf { typedef ModalMat<V, Shape<KIND>::NO, Shape<KIND>::NI> type; };
+template <typename V>
+struct MatOf<MK_SS, V> { typedef ModalSch<V> type; };
+
+// One element row of the march: modes of the element between node rows with
+// (x pair, z sum / difference) values q0 (lower) and q1, scaled by rho;
+// contributions to the lower (low) and upper (up) node row.
+template <int KIND, typename V>
+__device__ __forceinline__ void element(const typename MatOf<KIND, V>::type& K, const Pair<V> (&q0)[Shape<KIND>::NI][2],
+                                        const Pair<V> (&q1)[Shape<KIND>::NI][2], V rho,
+                                        Pair<V> (&low)[Shape<KIND>::NO][2], Pair<V> (&up)[Shape<KIND>::NO][2]) {
+  constexpr int NI = Shape<KIND>::NI, NO = Shape<KIND>::NO;
+  V u[NI][8], f[NO][8];
+#pragma unroll
+  for (int d = 0; d < NI; ++d)
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      const Pair<V> ys = padd(q1[d][z], q0[d][z]), yd = psub(q1[d][z], q0[d][z]);
+      u[d][4 * z] = sum_of(ys);
+      u[d][4 * z + 1] = dif_of(ys);
+      u[d][4 * z + 2] = sum_of(yd);
+      u[d][4 * z + 3] = dif_of(yd);
+    }
+  if constexpr (KIND == MK_SS) force_s<V>(K, u, f);
+  else force<NO, NI, Shape<KIND>::CO, V>(K, u, f);
+#pragma unroll
+  for (int c = 0; c < NO; ++c)
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      const Pair<V> fs = pmul(rho, mk<V>(z ? f[c][4] : V{}, f[c][4 * z + 1]));
+      const Pair<V> fd = pmul(rho, mk<V>(f[c][4 * z + 2], f[c][4 * z + 3]));
+      low[c][z] = psub(fs, fd);
+      up[c][z] = padd(fs, fd);
+    }
+}
+
+// ---- the march ------------------------------------------------------------------
+// IO supplies the inputs and takes the outputs of one load (offsets in bytes
+// from the start of a component plane):
+//   V    in(d, offset)          input component d at a node
+//   V    rho(offset)            element scale
+//   void fetch(pre, offset)     operands of a node's output
+//   void out(offset, acc, own, pre)   assembled values of the output components
+//                               and the node's own inputs
+template <int KIND, int RY, bool PF, typename V, typename IO>
+__device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, const IO& io, int nx, int ny, int nz,
+                                      int L) {
+  constexpr int NI = Shape<KIND>::NI, NO = Shape<KIND>::NO;
+  constexpr unsigned SZ = IO::kBytes;
+  const int lane = threadIdx.x & 31;
+  const int rl = nx + 2;
+  const int strips = (ny + RY - 1) / RY;
+  const int p0 = (int)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * kOut;
+  if (p0 >= strips * rl - 2) return;   // warp-uniform
+  const int p = min(p0 + lane, strips * rl - 1);
+  const int strip = p / rl;
+  const int xi = p - strip * rl - 1;
+  const bool vx = lane >= 1 && lane <= kOut && p0 + lane == p && xi >= 0 && xi < nx;
+  const int i = xi < 0 ? nx - 1 : (xi >= nx ? 0 : xi);
+  const int j0 = strip * RY;
+  // in-plane offsets of the node rows j0 - 1 .. j0 + RY (periodic); rows of
+  // the strip that this lane writes
+  unsigned ro[RY + 2];
+  bool ok[RY];
+#pragma unroll
+  for (int r = 0; r < RY + 2; ++r) {
+    int j = j0 - 1 + r;
+    j = j < 0 ? j + ny : j % ny;
+    ro[r] = (unsigned)(j * nx + i) * SZ;
+  }
+#pragma unroll
+  for (int r = 0; r < RY; ++r) ok[r] = vx && j0 + r < ny;
+  const unsigned nxy = (unsigned)(nx * ny) * SZ;
+  const int z0 = blockIdx.z * L;
+  const int Lc = min(L, nz - z0);
+  Pair<V> ps[RY + 2][NI];   // x sums and differences of the plane before
+  V own[RY][NI];            // its values on the strip's own rows
+  Pair<V> carry[RY][NO];    // contributions of the layer below to the plane before
+  unsigned zp = (unsigned)(z0 == 0 ? nz - 1 : z0 - 1) * nxy;   // the plane before
+#pragma unroll
+  for (int r = 0; r < RY + 2; ++r)
+#pragma unroll
+    for (int d = 0; d < NI; ++d) {
+      const V v = io.in(d, zp + ro[r]);
+      const V w = vdown(v);
+      ps[r][d] = mk<V>(vadd(w, v), vsub(w, v));
+    }
+#pragma unroll
+  for (int r = 0; r < RY; ++r) {
+#pragma unroll
+    for (int c = 0; c < NO; ++c) carry[r][c] = mk<V>(V{}, V{});
+#pragma unroll
+    for (int d = 0; d < NI; ++d) own[r][d] = V{};
+  }
+  unsigned zc = (unsigned)z0 * nxy;   // the plane above the layer
+  V vn[PF ? RY + 2 : 1][NI], rn[PF ? RY + 1 : 1];
+  if (PF) {
+#pragma unroll
+    for (int r = 0; r < RY + 2; ++r)
+#pragma unroll
+      for (int d = 0; d < NI; ++d) vn[PF ? r : 0][d] = io.in(d, zc + ro[r]);
+#pragma unroll
+    for (int r = 0; r < RY + 1; ++r) rn[PF ? r : 0] = io.rho(zp + ro[r]);
+  }
+#pragma unroll 1
+  for (int t = 0; t <= Lc; ++t) {
+    const unsigned zn = zc + nxy == nxy * (unsigned)nz ? 0 : zc + nxy;
+    V v[RY + 2][NI], rho[RY + 1];
+    typename IO::Pre pre[RY];
+    if (PF) {
+#pragma unroll
+      for (int r = 0; r < RY + 2; ++r)
+#pragma unroll
+        for (int d = 0; d < NI; ++d) {
+          v[r][d] = vn[PF ? r : 0][d];
+          vn[PF ? r : 0][d] = io.in(d, zn + ro[r]);
+        }
+#pragma unroll
+      for (int r = 0; r < RY + 1; ++r) {
+        rho[r] = rn[PF ? r : 0];
+        rn[PF ? r : 0] = io.rho(zc + ro[r]);
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < RY + 2; ++r)
+#pragma unroll
+        for (int d = 0; d < NI; ++d) v[r][d] = io.in(d, zc + ro[r]);
+#pragma unroll
+      for (int r = 0; r < RY + 1; ++r) rho[r] = io.rho(zp + ro[r]);
+    }
+    if (t > 0) {
+#pragma unroll
+      for (int r = 0; r < RY; ++r)
+        if (ok[r]) io.fetch(pre[r], zp + ro[r + 1]);
+    }
+    Pair<V> q0[NI][2], up[NO][2];
+#pragma unroll
+    for (int r = 0; r < RY + 2; ++r) {
+      Pair<V> q1[NI][2];
+#pragma unroll
+      for (int d = 0; d < NI; ++d) {
+        const V w = vdown(v[r][d]);
+        const Pair<V> x = mk<V>(vadd(w, v[r][d]), vsub(w, v[r][d]));
+        q1[d][0] = padd(x, ps[r][d]);
+        q1[d][1] = psub(x, ps[r][d]);
+        ps[r][d] = x;
+      }
+      if (r > 0) {
+        Pair<V> low[NO][2], un[NO][2];
+        element<KIND, V>(K, q0, q1, rho[r - 1], low, un);
+        if (r > 1) {
+          V acc[NO];
+#pragma unroll
+          for (int c = 0; c < NO; ++c) {
+            const Pair<V> ts = padd(up[c][0], low[c][0]), td = padd(up[c][1], low[c][1]);
+            const Pair<V> o = padd(carry[r - 2][c], psub(ts, td));
+            carry[r - 2][c] = padd(ts, td);
+            acc[c] = vadd(vsub(sum_of(o), dif_of(o)), vup(vadd(sum_of(o), dif_of(o))));
+          }
+          if (t > 0 && ok[r - 2]) io.out(zp + ro[r - 1], acc, own[r - 2], pre[r - 2]);
+#pragma unroll
+          for (int d = 0; d < NI; ++d) own[r - 2][d] = v[r - 1][d];
+        }
+#pragma unroll
+        for (int c = 0; c < NO; ++c) up[c][0] = un[c][0], up[c][1] = un[c][1];
+      }
+#pragma unroll
+      for (int d = 0; d < NI; ++d) q0[d][0] = q1[d][0], q0[d][1] = q1[d][1];
+    }
+    zp = zc;
+    zc = zn;
+  }
+}
+
+// ---- launch geometry -----------------------------------------------------------
+int sm_count();   // modal_f32.cu
+
+// Planes per chunk: the smallest waves x (planes + 2) for the warps that the
+// chip holds (a chunk evaluates one element layer and loads two node planes
+// more than it writes).
+inline int chunk_planes(int nz, i64 warps, int warps_per_sm) {
+  const i64 slots = (i64)sm_count() * warps_per_sm;
+  int best = nz;
+  const int most = nz < 4096 ? nz : 4096;   // grid z
+  double cost = 1e300;
+  for (int chunks = 1; chunks <= most; ++chunks) {
+    const int L = (nz + chunks - 1) / chunks;
+    if (chunks > 1 && L == (nz + chunks - 2) / (chunks - 1)) continue;
+    const i64 w = warps * ((nz + L - 1) / L);
+    const double c = (double)((w + slots - 1) / slots) * (L + 2.0);
+    if (c < cost) {
+      cost = c;
+      best = L;
+    }
+  }
+  return best;
+}
+
+// Grid (window groups, load groups, z chunks) and planes per chunk.
+inline dim3 grid_for(int nx, int ny, int nz, int groups, int rows, int blocks_per_sm, int* L) {
+  const i64 seq = (i64)((ny + rows - 1) / rows) * (nx + 2) - 2;   // positions between the first and last halo
+  const i64 windows = (seq + kOut - 1) / kOut;
+  const i64 blocks = (windows + kWarps - 1) / kWarps;
+  *L = chunk_planes(nz, blocks * kWarps * groups, blocks_per_sm * kWarps);
+  return dim3((unsigned)blocks, (unsigned)groups, (unsigned)((nz + *L - 1) / *L));
+}
+
+}  // namespace modal
+}  // namespace cell

@@ -1,0 +1,107 @@
+// Kernels and launchers of the modal operators for one scalar type (included
+// by modal_f32.cu and modal_f64.cu).
+#pragma once
+
+#include "modal.cuh"
+
+namespace cell {
+namespace modal {
+
+// Inputs and outputs of one load.
+template <int KIND, int MODE, typename T>
+struct IO {
+  static constexpr int NI = Shape<KIND>::NI, NO = Shape<KIND>::NO;
+  static constexpr bool kStep = MODE >= MM_STEP;
+  static constexpr bool kB = MODE != MM_APPLY;
+  static constexpr bool kXp = MODE == MM_STEP;
+  struct Pre {
+    T b[kB ? NO : 1], xp[kXp ? NO : 1], di[kStep ? NO : 1];
+  };
+  const T* x;
+  T* y;
+  const T* b;
+  const T* xp;
+  const T* dinv;
+  const T* rp;
+  i64 nn;
+  T c0, c1, c2;
+
+  // a warp-uniform base and a 32-bit byte offset (cell_setup admits at most
+  // 4e8 nodes: a component plane is below 2^32 bytes)
+  static constexpr unsigned kBytes = sizeof(T);
+  __device__ __forceinline__ static T ld(const T* p, i64 plane, unsigned o) {
+    return __ldg(reinterpret_cast<const T*>(reinterpret_cast<const char*>(p + plane) + o));
+  }
+  __device__ __forceinline__ T in(int d, unsigned o) const {
+    if (MODE == MM_PRE) return c0 * ld(dinv, d * nn, o) * ld(b, d * nn, o);
+    return ld(x, d * nn, o);
+  }
+  __device__ __forceinline__ T rho(unsigned o) const { return ld(rp, 0, o); }
+  __device__ __forceinline__ void fetch(Pre& p, unsigned o) const {
+#pragma unroll
+    for (int c = 0; c < NO; ++c) {
+      if (kB) p.b[c] = ld(b, c * nn, o);
+      if (kStep) p.di[c] = ld(dinv, c * nn, o);
+      // not through the read-only path: y may be xp (each node reads its own)
+      if (kXp) p.xp[c] = *reinterpret_cast<const T*>(reinterpret_cast<const char*>(xp + c * nn) + o);
+    }
+  }
+  __device__ __forceinline__ void out(unsigned o, T (&acc)[NO], const T (&own)[NI], const Pre& p) const {
+    if (KIND == MK_FULL) acc[NO - 1] = -acc[NO - 1];
+#pragma unroll
+    for (int c = 0; c < NO; ++c) {
+      T v;
+      if (MODE == MM_APPLY) {
+        v = acc[c];
+      } else if (MODE == MM_ADD) {
+        v = p.b[c] + acc[c];
+      } else if (MODE == MM_RESID) {
+        v = p.b[c] - acc[c];
+      } else {
+        const T x0 = own[c < NI ? c : 0];
+        v = x0 + c2 * p.di[c] * (p.b[c] - acc[c]);
+        if (MODE == MM_STEP) v += c1 * (x0 - p.xp[c]);
+        if (MODE == MM_STEP0) v += c1 * (x0 - c0 * p.di[c] * p.b[c]);
+        if (MODE == MM_PRE) v += c1 * x0;
+      }
+      *reinterpret_cast<T*>(reinterpret_cast<char*>(y + c * nn) + o) = v;
+    }
+  }
+};
+
+template <int KIND, int MODE, int RY, int MINB, bool PF, typename T>
+__global__ void __launch_bounds__(kThreads, MINB)
+k_modal(const ModalArgs<T> a, const __grid_constant__ typename MatOf<KIND, T>::type K, int L) {
+  const int r1 = min(a.nrhs, ((int)blockIdx.y + 1) * a.rg);
+#pragma unroll 1
+  for (int r = blockIdx.y * a.rg; r < r1; ++r) {
+    if (a.active && !a.active[r]) continue;
+    IO<KIND, MODE, T> io;
+    io.x = a.x + r * a.xs;
+    io.y = a.y + r * a.ys;
+    io.b = a.b + r * a.bs;
+    io.xp = a.xp + r * a.ps;
+    io.dinv = a.dinv;
+    io.rp = a.rho;
+    io.nn = (i64)a.nx * a.ny * a.nz;
+    io.c0 = io.c1 = io.c2 = T(0);
+    if (MODE >= MM_STEP) {
+      io.c1 = a.c12[0];
+      io.c2 = a.c12[1];
+    }
+    if (MODE == MM_STEP0 || MODE == MM_PRE) io.c0 = *a.c0;
+    march<KIND, RY, PF, T>(K, io, a.nx, a.ny, a.nz, L);
+  }
+}
+
+template <int KIND, int MODE, int RY, int MINB, bool PF, typename T>
+void launch(const ModalArgs<T>& a0, const typename MatOf<KIND, T>::type& K, cudaStream_t s) {
+  ModalArgs<T> a = a0;
+  if (a.rg < 1) a.rg = 1;
+  int L = 0;
+  const dim3 grid = grid_for(a.nx, a.ny, a.nz, (a.nrhs + a.rg - 1) / a.rg, RY, MINB, &L);
+  note_launch(), k_modal<KIND, MODE, RY, MINB, PF, T><<<grid, kThreads, 0, s>>>(a, K, L);
+}
+
+}  // namespace modal
+}  // namespace cell
