@@ -101,12 +101,13 @@ typedef struct cell_options {
   int coarse_dofs;     /* stop coarsening once a level has at most this many dofs */
   int load_mask;       /* bit I set = solve load I (default 0x1FF = all nine) */
   int profile;         /* nonzero: time kernel classes with CUDA events (cell_stats) */
-  int tensor_cores;    /* MIXED: 0 = SIMT FP32 applies only; 1 (default) = fine-grid smoothing
-                          applies of both preconditioner blocks (A and Sbar) on tcgen05
-                          tensor cores: node-centric TF32 element contraction with FP32
-                          accumulation, any grid size; 2 = also the Krylov operator Ahat
-                          (3xTF32 split, FP32-accurate), used where nx % 16 == 0,
-                          ny % 4 == 0, nz % 2 == 0. */
+  int tensor_cores;    /* MIXED: 0 = SIMT FP32 applies only; 1 (default) = for materials without
+                          the mm2 mirror planes, fine-grid smoothing applies of both
+                          preconditioner blocks (A and Sbar) on tcgen05 tensor cores:
+                          node-centric TF32 element contraction with FP32 accumulation, any
+                          grid size (mm2 materials smooth in FP32 with the modal operators,
+                          which are faster); 2 = also the Krylov operator Ahat (3xTF32 split,
+                          FP32-accurate), used where nx % 16 == 0, ny % 4 == 0, nz % 2 == 0. */
   int const_bank;      /* MIXED: nonzero (default) = FP32 element matrices in one of 4
                           library-wide __constant__ slots (shared by handles with equal
                           matrices), falling back to kernel parameters if all are taken */
@@ -130,8 +131,9 @@ typedef struct cell_options {
                           length) on this GPU and grid and keep the fastest per block (cell_stats
                           reports them); every tile gives bitwise the same result.  0 = widest
                           tile and a wave-count heuristic.  MIXED (any tensor_cores): nonzero also
-                          times the coarse levels' stencil apply with 1, 3 and 9 loads per thread
-                          and keeps the fastest per level (bitwise-neutral; cell_stats.stencil_rg). */
+                          times the coarse levels' operator with 1, 3 and 9 loads per thread
+                          (mm2 materials: per block, one after another) and keeps the fastest
+                          per level (bitwise-neutral; cell_stats.stencil_rg). */
 } cell_options;
 
 typedef enum cell_precond {
@@ -184,10 +186,10 @@ typedef struct cell_stats {
                                        A, [1] Schur Sbar): x width in nodes and z-chunk length;
                                        0 = not tuned (default tile or SIMT path) */
   double tc_tile_us[2];             /* the tuned tile's time per 9-load Chebyshev launch, us */
-  int stencil_rg[2][8];             /* MIXED: loads per thread of the coarse stencil apply per
-                                       multigrid level ([0] elastic, [1] Schur; level 0 = fine
-                                       grid, always 0); 0 = size default, 1/3/9 = tuned at set-up
-                                       (options.autotune; bitwise-neutral) */
+  int stencil_rg[2][8];             /* MIXED: loads per thread (mm2 materials: per block) of the
+                                       coarse operator per multigrid level ([0] elastic, [1]
+                                       Schur; level 0 = fine grid, always 0); 0 = size default,
+                                       1/3/9 = tuned at set-up (options.autotune; bitwise-neutral) */
 } cell_stats;
 
 typedef struct cell_handle cell_handle;
@@ -363,8 +365,8 @@ int cell_apply(cell_handle* h, const void* x, void* y, int nrhs, int dtype);
  * S0 = C_e + B_e (A_e + shift I)^-1 B_e^T, 1 component).  x, y: device,
  * nrhs vectors of [comp][node] (3nn or nn values each), not aliased.
  * dtype CELL_F32 / CELL_F64: SIMT; CELL_F32_TC: the node-centric tensor-core
- * kernel used by the smoothers (TF32 inputs, FP32 accumulation; any grid
- * size).  Asynchronous on the handle's stream. */
+ * kernel of the smoothers of non-mm2 materials (TF32 inputs, FP32
+ * accumulation; any grid size).  Asynchronous on the handle's stream. */
 int cell_apply_block(cell_handle* h, int block, const void* x, void* y, int nrhs, int dtype);
 
 /* Set the CTA tile of the tensor-core smoother of one block (cell_block) for
@@ -380,13 +382,14 @@ int cell_apply_block(cell_handle* h, int block, const void* x, void* y, int nrhs
  * or a grid it does not support). */
 int cell_set_tile(cell_handle* h, int block, int xt, int L);
 
-/* Set the loads per thread (rg = 1, 3 or 9; 0 = the size default) of the
- * assembled-stencil apply on multigrid level `level` (>= 1) of one block
+/* Set the loads per thread (mm2 materials: per block, one after another; rg =
+ * 1, 3 or 9; 0 = the size default) of the operator on multigrid level `level` (>= 1) of one block
  * (cell_block), replacing the value cell_setup tuned.  Results do not depend
  * on rg (every (node, load) runs the same operation sequence); it changes
  * launch geometry and speed only.  Takes effect for later launches; a solve
  * graph captured before the call keeps the value it was captured with.
- * Levels small enough for the four-lane stencil kernel ignore it.  Errors:
+ * Levels of at most 4096 nodes are not tuned, and the four-lane stencil kernel
+ * (other materials) ignores it there.  Errors:
  * CELL_EINVAL for a null handle, an unknown block, a level outside
  * 1 .. levels-1, an rg not in {0, 1, 3, 9}, or FP64 precision. */
 int cell_set_stencil_rg(cell_handle* h, int block, int level, int rg);

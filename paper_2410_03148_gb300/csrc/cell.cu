@@ -197,6 +197,13 @@ struct Level {
   T* dense = nullptr;    // coarsest: regularised inverse (n x n, symmetric)
   int ndense = 0;
   bool coarsest = false;
+  // mm2 materials: rediscretised level (operator from its own rho, no stencil)
+  const T* rho = nullptr;   // element scales of this level
+  const T* di = nullptr;    // 1 / (rho summed around a node)
+  T dk[3] = {0, 0, 0};      // inverse element diagonal per component
+  cell::ModalMat<T, 3, 3> uu;
+  cell::ModalSch<T> ss;
+  std::vector<double> kb;   // element matrix of the block (coarsest level: dense assembly)
 };
 
 template <typename T>
@@ -254,6 +261,7 @@ struct cell_handle {
   bool modal = false;            // mm2 material: operators in modal form
   ModalSet<float> m32;
   ModalSet<double> m64;
+  std::vector<void*> rho_lv, di_lv;   // per multigrid level (solver precision): element scales, inverse diagonals
   cell::ModalMat<cell::DF, 4, 4> mdf;
   Arena arena;
   float* rho32 = nullptr;
@@ -419,9 +427,12 @@ int assemble_dense(cell_handle* h, BlockMG<T>& mg, int l, std::vector<double>& A
   const i64 nn = L.nn;
   const int n = (int)(NC * nn);
   A.assign((size_t)n * n, 0.0);
-  std::vector<T> ke;
+  std::vector<T> ke, rl;
   std::vector<double> rho;
-  if (l == 0) {
+  if (h->modal) {
+    rl.resize(nn);
+    CK(cudaMemcpyAsync(rl.data(), L.rho, nn * sizeof(T), cudaMemcpyDeviceToHost, h->st));
+  } else if (l == 0) {
     rho.resize(nn);
     CK(cudaMemcpyAsync(rho.data(), h->rho64, nn * sizeof(double), cudaMemcpyDeviceToHost, h->st));
   } else {
@@ -439,7 +450,8 @@ int assemble_dense(cell_handle* h, BlockMG<T>& mg, int l, std::vector<double>& A
         for (int b = 0; b < 8; ++b)
           for (int dd = 0; dd < NC; ++dd) {
             const int entry = (a * NC + c) * R + b * NC + dd;
-            const double v = l == 0 ? rho[e] * mg.fixed_host[entry] : (double)ke[(size_t)entry * nn + e];
+            const double v = h->modal ? (double)rl[e] * L.kb[entry]
+                                      : (l == 0 ? rho[e] * mg.fixed_host[entry] : (double)ke[(size_t)entry * nn + e]);
             A[(size_t)(c * nn + node[a]) * n + dd * nn + node[b]] += v;
           }
   }
@@ -540,6 +552,48 @@ int alloc_mg(cell_handle* h, BlockMG<T>& mg, const double* fixed_block) {
   return CELL_OK;
 }
 
+// (0, 1 / theta), then (c1_k, c2_k), k = 1 .. deg - 1, for the interval
+// [cheb_lo, 1] x cheb_hi x lmax.
+template <typename T>
+void cheb_coefficients(double lmax, const cell_options& o, int deg, T* c) {
+  const double hi = lmax * o.cheb_hi, lo = hi * o.cheb_lo;
+  const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
+  c[0] = T(0);
+  c[1] = (T)(1.0 / theta);
+  double rp = 1.0 / sigma;
+  for (int k = 1; k < deg; ++k) {
+    const double rk = 1.0 / (2.0 * sigma - rp);
+    c[2 * k] = (T)(rk * rp);
+    c[2 * k + 1] = (T)(2.0 * rk / delta);
+    rp = rk;
+  }
+}
+
+// Regularised inverse of the coarsest level's operator (null space:
+// componentwise constants), if the level has one.
+template <typename T, int NC>
+int dense_inverse(cell_handle* h, BlockMG<T>& mg) {
+  Level<T>& Lc = mg.lv.back();
+  if (!Lc.dense) return CELL_OK;
+  const i64 n = Lc.ndense;
+  std::vector<double> A;
+  CKS((assemble_dense<T, NC>(h, mg, (int)mg.lv.size() - 1, A)));  // synchronises the stream
+  double tr = 0.0;
+  for (i64 i = 0; i < n; ++i) tr += A[(size_t)i * n + i];
+  const double alpha = tr / (double)n;
+  for (int c = 0; c < NC; ++c)
+    for (i64 p = 0; p < Lc.nn; ++p)
+      for (i64 q = 0; q < Lc.nn; ++q) A[(size_t)(c * Lc.nn + p) * n + c * Lc.nn + q] += alpha / (double)Lc.nn;
+  if (cellhost::spd_inverse(A.data(), (int)n) != 0) {
+    set_error("coarsest multigrid level is not positive definite (rho must be > 0)");
+    return CELL_EINVAL;
+  }
+  mg.dense_host.resize(A.size());
+  for (size_t i = 0; i < A.size(); ++i) mg.dense_host[i] = (T)A[i];
+  CK(cudaMemcpyAsync(Lc.dense, mg.dense_host.data(), mg.dense_host.size() * sizeof(T), cudaMemcpyHostToDevice, h->st));
+  return CELL_OK;
+}
+
 // Numerics of the hierarchy for the handle's current rho (every design):
 // Galerkin coarse element matrices, stencils, Jacobi diagonals, Chebyshev
 // bounds and the coarsest regularised inverse.
@@ -562,27 +616,7 @@ int fill_mg(cell_handle* h, BlockMG<T>& mg) {
   }
   std::vector<unsigned> bits(nl, 0u);
   CK(cudaMemcpyAsync(bits.data(), mg.lbits, nl * sizeof(unsigned), cudaMemcpyDeviceToHost, h->st));
-  Level<T>& Lc = mg.lv.back();
-  if (Lc.dense) {
-    const i64 n = Lc.ndense;
-    std::vector<double> A;
-    CKS((assemble_dense<T, NC>(h, mg, nl - 1, A)));  // synchronises the stream
-    // regularise the null space (componentwise constants) and invert
-    double tr = 0.0;
-    for (i64 i = 0; i < n; ++i) tr += A[(size_t)i * n + i];
-    const double alpha = tr / (double)n;
-    for (int c = 0; c < NC; ++c)
-      for (i64 p = 0; p < Lc.nn; ++p)
-        for (i64 q = 0; q < Lc.nn; ++q) A[(size_t)(c * Lc.nn + p) * n + c * Lc.nn + q] += alpha / (double)Lc.nn;
-    if (cellhost::spd_inverse(A.data(), (int)n) != 0) {
-      set_error("coarsest multigrid level is not positive definite (rho must be > 0)");
-      return CELL_EINVAL;
-    }
-    mg.dense_host.resize(A.size());
-    for (size_t i = 0; i < A.size(); ++i) mg.dense_host[i] = (T)A[i];
-    CK(cudaMemcpyAsync(Lc.dense, mg.dense_host.data(), mg.dense_host.size() * sizeof(T),
-                       cudaMemcpyHostToDevice, h->st));
-  }
+  CKS((dense_inverse<T, NC>(h, mg)));
   CK(cudaStreamSynchronize(h->st));
   for (int l = 1; l < nl; ++l) {
     float lf;
@@ -592,18 +626,7 @@ int fill_mg(cell_handle* h, BlockMG<T>& mg) {
   const cell_options& o = h->d.opt;
   const size_t stride = mg.cc_host.size() / nl;
   for (int l = 0; l < nl; ++l) {
-    const double hi = mg.lv[l].lmax * o.cheb_hi, lo = hi * o.cheb_lo;
-    const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
-    T* c = mg.cc_host.data() + stride * l;
-    c[0] = T(0);
-    c[1] = (T)(1.0 / theta);
-    double rp = 1.0 / sigma;
-    for (int k = 1; k < mg.lv[l].deg; ++k) {
-      const double rk = 1.0 / (2.0 * sigma - rp);
-      c[2 * k] = (T)(rk * rp);
-      c[2 * k + 1] = (T)(2.0 * rk / delta);
-      rp = rk;
-    }
+    cheb_coefficients(mg.lv[l].lmax, o, mg.lv[l].deg, mg.cc_host.data() + stride * l);
   }
   CK(cudaMemcpyAsync(mg.cc_dev, mg.cc_host.data(), mg.cc_host.size() * sizeof(T), cudaMemcpyHostToDevice,
                      h->st));
@@ -669,12 +692,230 @@ void vcycle(cell_handle* h, BlockMG<T>& mg, int l, const T* b, i64 bs, T* x, i64
   else cell::axpy_view<T, NC>(x, xs, d, ws, L.nn, 9, mask, h->st);
 }
 
+// ---------------------------------------------------------------------------
+// multigrid on rediscretised levels (mm2 materials)
+// ---------------------------------------------------------------------------
+
+// Sizes of the next coarser grid: every axis within 0.7 of the longest one is
+// (about) halved, so elements become cubes before the other axes follow.
+// Returns false if nothing can be coarsened.
+bool coarser(const int n[3], int c[3]) {
+  const int m = std::max(n[0], std::max(n[1], n[2]));
+  bool any = false;
+  for (int d = 0; d < 3; ++d) {
+    const bool half = n[d] >= 3 && 10 * n[d] >= 7 * m;
+    c[d] = half ? (n[d] + 1) / 2 : n[d];
+    any = any || half;
+  }
+  return any;
+}
+
+// Element matrix of a preconditioner block (A: 24 x 24, Sbar or C: 8 x 8) on a
+// grid of n nodes per axis.
+int block_matrix(const cell_handle* h, const int n[3], int nc, std::vector<double>& M) {
+  double K[1024], S[64];
+  const double hh[3] = {1.0 / n[0], 1.0 / n[1], 1.0 / n[2]};
+  cellhost::element_matrix(h->Cn, h->en, h->kn, hh, K);
+  const int R = 8 * nc;
+  M.resize(R * R);
+  if (nc == 3) {
+    for (int a = 0; a < 8; ++a)
+      for (int c = 0; c < 3; ++c)
+        for (int b = 0; b < 8; ++b)
+          for (int d = 0; d < 3; ++d) M[(a * 3 + c) * R + b * 3 + d] = K[(4 * a + c) * 32 + 4 * b + d];
+    return CELL_OK;
+  }
+  if (h->d.opt.precond == CELL_PRECOND_DBP) {
+    for (int a = 0; a < 8; ++a)
+      for (int b = 0; b < 8; ++b) M[a * 8 + b] = -K[(4 * a + 3) * 32 + 4 * b + 3];
+    return CELL_OK;
+  }
+  if (cellhost::local_schur(K, h->d.opt.schur_shift, S) != 0) {
+    set_error("elastic element block is not positive definite (check C)");
+    return CELL_EINVAL;
+  }
+  std::copy(S, S + 64, M.begin());
+  return CELL_OK;
+}
+
+template <typename T, int NC>
+int alloc_mg_modal(cell_handle* h, BlockMG<T>& mg) {
+  const cell_options& o = h->d.opt;
+  const int R = 8 * NC;
+  mg.nc = NC;
+  mg.lv.clear();
+  int n[3] = {h->nx, h->ny, h->nz};
+  for (;;) {
+    Level<T> L;
+    L.nx = n[0];
+    L.ny = n[1];
+    L.nz = n[2];
+    L.nn = (i64)n[0] * n[1] * n[2];
+    CKS(block_matrix(h, n, NC, L.kb));
+    L.lmax = cellhost::jacobi_lmax(L.kb.data(), R);
+    for (int c = 0; c < NC; ++c) L.dk[c] = (T)(1.0 / L.kb[c * R + c]);
+    std::vector<double> Km(R * R);
+    cellhost::modal_matrix(L.kb.data(), NC, Km.data());
+    if constexpr (NC == 3) fill_modal<3, 3, T>(Km.data(), 3, 0, L.uu, [](double v) { return (T)v; });
+    else
+      for (int m = 0; m < 8; ++m) L.ss.s[m] = (T)Km[m * 8 + m];
+    // scales and diagonals, shared by the two blocks (the grids are the same)
+    const size_t l = mg.lv.size();
+    if (h->di_lv.size() <= l) {
+      T *r = nullptr, *di = nullptr;
+      if (l > 0) CKS(h->arena.alloc(&r, L.nn));
+      CKS(h->arena.alloc(&di, L.nn));
+      h->rho_lv.push_back(r);
+      h->di_lv.push_back(di);
+    }
+    L.rho = l == 0 ? rho_of<T>(h) : static_cast<T*>(h->rho_lv[l]);
+    L.di = static_cast<T*>(h->di_lv[l]);
+    const size_t wn = (size_t)9 * NC * L.nn;
+    if (l > 0) {
+      CKS(h->arena.alloc(&L.b, wn));
+      CKS(h->arena.alloc(&L.x, wn));
+    }
+    CKS(h->arena.alloc(&L.r, wn));
+    CKS(h->arena.alloc(&L.d, wn));
+    mg.lv.push_back(L);
+    int c[3];
+    if (L.nn * NC <= (i64)o.coarse_dofs || !coarser(n, c)) break;
+    std::copy(c, c + 3, n);
+  }
+  Level<T>& Lc = mg.lv.back();
+  Lc.coarsest = true;
+  const i64 nd = NC * Lc.nn;
+  if (nd <= 3000) {
+    CKS(h->arena.alloc(&Lc.dense, (size_t)nd * nd));
+    Lc.ndense = (int)nd;
+  }
+  // Chebyshev coefficients (the bounds do not depend on the design): (0, 1 / theta),
+  // then (c1_k, c2_k)
+  const int nl = (int)mg.lv.size();
+  const int degc = std::max(8, 4 * o.cheb_degree);
+  const size_t stride = 2 * (degc + 1);
+  CKS(h->arena.alloc(&mg.cc_dev, stride * nl));
+  mg.cc_host.assign(stride * nl, T(0));
+  for (int l = 0; l < nl; ++l) {
+    Level<T>& L = mg.lv[l];
+    L.cc = mg.cc_dev + stride * l;
+    L.deg = (L.coarsest && !L.dense) ? degc : o.cheb_degree;
+    cheb_coefficients(L.lmax, o, L.deg, mg.cc_host.data() + stride * l);
+  }
+  CK(cudaMemcpyAsync(mg.cc_dev, mg.cc_host.data(), mg.cc_host.size() * sizeof(T), cudaMemcpyHostToDevice, h->st));
+  return CELL_OK;
+}
+
+template <typename T>
+cell::GridPair grid_pair(const Level<T>& F, const Level<T>& C) {
+  return cell::GridPair{{F.nx, F.ny, F.nz}, {C.nx, C.ny, C.nz}};
+}
+
+// Numerics of both hierarchies for the current rho: scales and diagonals of
+// every level, the coarsest inverses.
+template <typename T>
+int fill_mg_modal(cell_handle* h) {
+  Krylov<T>& K = kry<T>(h);
+  const std::vector<Level<T>>& lv = K.mgu.lv.size() >= K.mgp.lv.size() ? K.mgu.lv : K.mgp.lv;
+  for (size_t l = 0; l < lv.size(); ++l) {
+    if (l > 0) cell::mg_rho<T>(lv[l - 1].rho, static_cast<T*>(h->rho_lv[l]), grid_pair(lv[l - 1], lv[l]), h->st);
+    cell::mg_dinv<T>(lv[l].rho, static_cast<T*>(h->di_lv[l]), lv[l].nx, lv[l].ny, lv[l].nz, h->st);
+  }
+  CKS((dense_inverse<T, 3>(h, K.mgu)));
+  CKS((dense_inverse<T, 1>(h, K.mgp)));
+  return CELL_OK;
+}
+
+// One launch of a level's operator.
+template <typename T, int NC>
+void modal_level(cell_handle* h, BlockMG<T>& mg, int l, int mode, const T* x, i64 xs, T* y, i64 ys, const T* b, i64 bs,
+                 const T* xp, i64 ps, const T* c12, const int* mask) {
+  Level<T>& L = mg.lv[l];
+  cell::ModalArgs<T> m{};
+  m.x = x; m.xs = xs; m.y = y; m.ys = ys; m.b = b; m.bs = bs; m.xp = xp; m.ps = ps;
+  m.dinv = L.di; m.rho = L.rho; m.c12 = c12; m.c0 = L.cc + 1;
+  for (int c = 0; c < NC; ++c) m.dk[c] = L.dk[c];
+  m.nx = L.nx; m.ny = L.ny; m.nz = L.nz;
+  m.nrhs = 9; m.active = mask; m.rg = L.rg;
+  const int pcls = l > 0 ? CELL_PROF_COARSE : (NC == 3 ? CELL_PROF_ELASTIC0 : CELL_PROF_SCHUR0);
+  const int ip = h->prof.begin(h->st, pcls);
+  if constexpr (NC == 3) cell::modal_uu<T>(m, L.uu, mode, h->st);
+  else cell::modal_ss<T>(m, L.ss, mode, h->st);
+  h->prof.end(pcls, ip, h->st);
+}
+
+// x = V-cycle approximation of A_l^-1 b (zero initial guess).  Chebyshev
+// smoothing in three-term form: an iterate alternates between x and the
+// level's scratch, every step one launch that reads b and two iterates and
+// writes one (the direction form moved a third more and needed separate
+// start and end passes).
+template <typename T, int NC>
+void vcycle_modal(cell_handle* h, BlockMG<T>& mg, int l, const T* b, i64 bs, T* x, i64 xs, const int* mask) {
+  Level<T>& L = mg.lv[l];
+  const i64 ws = NC * L.nn;
+  if (L.coarsest && L.dense) {
+    cell::dense_solve<T>(L.dense, L.ndense, b, bs, x, xs, L.nn, NC, 9, mask, h->st);
+    return;
+  }
+  const int deg = L.deg;
+  // the buffer that holds the iterate between pre- and post-smoothing: the
+  // deg post-smoothing steps alternate and the last one writes x
+  const bool in_x = L.coarsest || deg % 2 == 0;
+  T* P = in_x ? x : L.d;
+  T* Q = in_x ? L.d : x;
+  const i64 psd = in_x ? xs : ws, qsd = in_x ? ws : xs;
+  // pre-smoothing from zero: steps 1 .. deg - 1, the last one writes P
+  if (deg == 1) {
+    cell::mg_scale<T, NC>(b, bs, P, psd, L.di, L.dk, L.cc + 1, L.nn, 9, mask, h->st);
+  } else {
+    const T* cur = nullptr;
+    i64 cs = 0;
+    for (int k = 1; k < deg; ++k) {
+      const bool toP = (deg - 1 - k) % 2 == 0;
+      T* y = toP ? P : Q;
+      const i64 ysd = toP ? psd : qsd;
+      const int mode = k == 1 ? cell::MM_PRE : (k == 2 ? cell::MM_STEP0 : cell::MM_STEP);
+      modal_level<T, NC>(h, mg, l, mode, cur, cs, y, ysd, b, bs, y, ysd, L.cc + 2 * k, mask);
+      cur = y;
+      cs = ysd;
+    }
+  }
+  if (L.coarsest) return;
+  Level<T>& C = mg.lv[l + 1];
+  const i64 cws = NC * C.nn;
+  modal_level<T, NC>(h, mg, l, cell::MM_RESID, P, psd, L.r, ws, b, bs, nullptr, 0, L.cc, mask);
+  const cell::GridPair g = grid_pair(L, C);
+  cell::mg_restrict<T, NC>(L.r, ws, C.b, cws, g, 9, mask, h->st);
+  vcycle_modal<T, NC>(h, mg, l + 1, C.b, cws, C.x, cws, mask);
+  cell::mg_prolong<T, NC>(C.x, cws, P, psd, g, 9, mask, h->st);
+  // post-smoothing
+  const T* cur = P;
+  i64 cs = psd;
+  for (int k = 0; k < deg; ++k) {
+    T* y = k % 2 == 0 ? Q : P;
+    const i64 ysd = k % 2 == 0 ? qsd : psd;
+    modal_level<T, NC>(h, mg, l, k == 0 ? cell::MM_POST : cell::MM_STEP, cur, cs, y, ysd, b, bs, y, ysd, L.cc + 2 * k,
+                       mask);
+    cur = y;
+    cs = ysd;
+  }
+}
+
 // k V-cycles by residual correction: x ~ A^-1 b.
 template <typename T, int NC>
 void block_solve(cell_handle* h, BlockMG<T>& mg, int cycles, const T* b, i64 bs, T* x, i64 xs,
                  T* rwork, T* ework, const int* mask) {
-  vcycle<T, NC>(h, mg, 0, b, bs, x, xs, mask);
   const i64 ws = NC * h->nn;
+  if (h->modal) {
+    vcycle_modal<T, NC>(h, mg, 0, b, bs, x, xs, mask);
+    for (int c = 1; c < cycles; ++c) {
+      modal_level<T, NC>(h, mg, 0, cell::MM_RESID, x, xs, rwork, ws, b, bs, nullptr, 0, mg.lv[0].cc, mask);
+      vcycle_modal<T, NC>(h, mg, 0, rwork, ws, ework, ws, mask);
+      cell::axpy_view<T, NC>(x, xs, ework, ws, h->nn, 9, mask, h->st);
+    }
+    return;
+  }
+  vcycle<T, NC>(h, mg, 0, b, bs, x, xs, mask);
   for (int c = 1; c < cycles; ++c) {
     cell::ApplyArgs<T> a{};
     a.x = x; a.xs = xs; a.y = rwork; a.ys = ws; a.b = b; a.bs = bs; a.alpha = T(-1); a.beta = T(1);
@@ -782,6 +1023,11 @@ int setup_krylov(cell_handle* h) {
     CKS(h->arena.alloc(&K.rp, (size_t)9 * h->nn));
     CKS(h->arena.alloc(&K.ep, (size_t)9 * h->nn));
   }
+  if (h->modal) {
+    CKS((alloc_mg_modal<T, 3>(h, K.mgu)));
+    CKS((alloc_mg_modal<T, 1>(h, K.mgp)));
+    return CELL_OK;
+  }
   // level-0 blocks of the preconditioner: A_e (24x24 u-block of K0), S0
   std::vector<double> Auu(576);
   for (int a = 0; a < 8; ++a)
@@ -795,6 +1041,7 @@ int setup_krylov(cell_handle* h) {
 
 template <typename T>
 int fill_krylov(cell_handle* h) {
+  if (h->modal) return fill_mg_modal<T>(h);
   Krylov<T>& K = kry<T>(h);
   CKS((fill_mg<T, 3>(h, K.mgu)));
   CKS((fill_mg<T, 1>(h, K.mgp)));
@@ -1585,10 +1832,11 @@ int tune_tiles(cell_handle* h) {
     Level<float>& L0 = kind == cell::NK_UU ? K.mgu.lv[0] : K.mgp.lv[0];
     const i64 ws = (kind == cell::NK_UU ? 3 : 1) * h->nn;
     cell::ApplyArgs<float> a{};
-    a.x = L0.d; a.xs = ws; a.y = L0.r; a.ys = ws; a.sol = K.V; a.ss = ws; a.dout = L0.d2; a.ds = ws;
+    a.x = L0.d; a.xs = ws; a.y = L0.r; a.ys = ws; a.sol = K.V; a.ss = ws;
+    a.dout = h->modal ? K.V + 9 * ws : L0.d2; a.ds = ws;
     a.cc = L0.cc; a.sol_zero = 0;
     a.nx = h->nx; a.ny = h->ny; a.nz = h->nz;
-    a.dinv = L0.dinv; a.rho = K.rho; a.cslot1 = h->cslot1;
+    a.dinv = h->modal ? K.V + 18 * ws : L0.dinv; a.rho = K.rho; a.cslot1 = h->cslot1;
     h->nct[kind] = cell::nc_autotune(kind, a, h->ncb + cell::nc_table_floats() * kind, cell::AM_CHEB, 9,
                                      h->tc_err, h->st, &h->nct_us[kind]);
   }
@@ -1599,14 +1847,55 @@ int tune_tiles(cell_handle* h) {
   return CELL_OK;
 }
 
+// Loads per block (one after another) of a rediscretised level's operator, timed
+// at set-up on the level's scratch vectors: 1, 3 or 9, bitwise-neutral.  Levels
+// of at most 4096 nodes keep 1 (they do not fill the chip).
+template <typename T, int NC>
+void tune_modal(cell_handle* h, BlockMG<T>& mg, int l) {
+  constexpr int kReps = 3;
+  Level<T>& L = mg.lv[l];
+  if (L.nn <= 4096) return;
+  const i64 ws = NC * L.nn;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+    if (e0) cudaEventDestroy(e0);
+    return;
+  }
+  int best = 0;
+  float best_t = 3.0e38f;
+  for (int rg : {1, 3, 9}) {
+    L.rg = rg;
+    auto step = [&] {
+      modal_level<T, NC>(h, mg, l, cell::MM_STEP, L.b, ws, L.d, ws, L.r, ws, L.x, ws, L.cc, nullptr);
+    };
+    step();
+    cudaEventRecord(e0, h->st);
+    for (int r = 0; r < kReps; ++r) step();
+    cudaEventRecord(e1, h->st);
+    float ms = 0.f;
+    if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) continue;
+    if (ms < best_t) {
+      best_t = ms;
+      best = rg;
+    }
+  }
+  L.rg = best;
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+}
+
 // Loads per thread of every coarse level's stencil apply, timed at set-up in
 // the Chebyshev mode on the level's own scratch vectors (bitwise-neutral).
 template <typename T, int NC>
 void tune_stencils(cell_handle* h, BlockMG<T>& mg) {
   for (size_t l = 1; l < mg.lv.size(); ++l) {
     Level<T>& L = mg.lv[l];
-    if (!L.st || L.dense) continue;
+    if (L.dense) continue;
     const i64 ws = NC * L.nn;
+    if (h->modal) {
+      tune_modal<T, NC>(h, mg, (int)l);
+      continue;
+    }
     cell::ApplyArgs<T> a{};
     a.x = L.d; a.xs = ws; a.y = L.r; a.ys = ws; a.sol = L.x; a.ss = ws; a.dout = L.d2; a.ds = ws;
     a.dinv = L.dinv; a.cc = L.cc; a.st = L.st;

@@ -104,6 +104,9 @@ enum ModalMode {
   MM_RESID = 2,   // y = b - A x
   // Chebyshev-Jacobi steps on A x = b in three-term form, D = diag(A):
   //   x_{k+1} = x_k + c1 (x_k - x_{k-1}) + c2 D^-1 (b - A x_k)
+  // With the mirror planes every corner of an element has the same diagonal
+  // entry k_c of component c, so D^-1 = dk[c] * dinv with dk[c] = 1 / k_c and
+  // dinv = 1 / (sum of the 8 rho around the node).
   MM_STEP = 3,    // y = x_{k+1}, x_{k-1} = xp (y may be xp)
   MM_STEP0 = 4,   // the same with x_{k-1} = c0 D^-1 b
   MM_PRE = 5,     // the same with x_k = c0 D^-1 b (not stored) and x_{k-1} = 0
@@ -132,7 +135,8 @@ struct ModalArgs {
   T* y; i64 ys;            // output
   const T* b; i64 bs;      // right-hand side (all modes but MM_APPLY)
   const T* xp; i64 ps;     // MM_STEP: x_{k-1}
-  const T* dinv;           // inverse diagonal [NC][nn] (steps)
+  const T* dinv;           // steps: 1 / (rho summed around the node), [nn]
+  T dk[3];                 // steps: inverse element diagonal per component
   const T* rho;            // element scales
   const T* c12;            // device (c1, c2) of the step
   const T* c0;             // device c0 of the first step (MM_STEP0, MM_PRE)
@@ -238,6 +242,27 @@ bool apply_nc(int kind, const ApplyArgs<float>& a, const float* Btab, int mode, 
 // *best_us (if non-null) = its time per launch in microseconds.
 NcTile nc_autotune(int kind, const ApplyArgs<float>& a, const float* Btab, int mode, int nrhs, int* err,
                    cudaStream_t s, float* best_us);
+
+// Transfers between a grid of nf nodes per axis and a coarse one of nc nodes
+// (nc[d] = nf[d] or about half of it, any ratio up to 2): periodic grids of
+// the same cell, trilinear interpolation at the true positions, restriction =
+// its transpose.
+struct GridPair {
+  int nf[3], nc[3];
+};
+// xf += P xc (loads masked)
+template <typename T, int NC> void mg_prolong(const T* xc, i64 cs, T* xf, i64 fs, const GridPair& g, int nrhs,
+                                              const int* active, cudaStream_t s);
+// bc = P^T rf
+template <typename T, int NC> void mg_restrict(const T* rf, i64 rs, T* bc, i64 cs, const GridPair& g, int nrhs,
+                                               const int* active, cudaStream_t s);
+// element scales of the coarse grid: means over the overlapped fine elements
+template <typename T> void mg_rho(const T* rf, T* rc, const GridPair& g, cudaStream_t s);
+// dinv = 1 / (rho summed over the 8 elements around a node)
+template <typename T> void mg_dinv(const T* rho, T* dinv, int nx, int ny, int nz, cudaStream_t s);
+// x = c0 dk[c] dinv b (a first Chebyshev step from zero)
+template <typename T, int NC> void mg_scale(const T* b, i64 bs, T* x, i64 xs, const T* dinv, const T* dk, const T* c0,
+                                            i64 nn, int nrhs, const int* active, cudaStream_t s);
 
 // ---- multigrid helpers (mg.cu) ----------------------------------------------
 // r = b, d = c2 Dinv b with c2 read from device memory (*c2p)

@@ -15,7 +15,7 @@ struct IO {
   static constexpr bool kB = MODE != MM_APPLY;
   static constexpr bool kXp = MODE == MM_STEP;
   struct Pre {
-    T b[kB ? NO : 1], xp[kXp ? NO : 1], di[kStep ? NO : 1];
+    T b[kB ? NO : 1], xp[kXp ? NO : 1], di;
   };
   const T* x;
   T* y;
@@ -24,7 +24,8 @@ struct IO {
   const T* dinv;
   const T* rp;
   i64 nn;
-  T c0, c1, c2;
+  T c1;
+  T k0[3], k2[3];   // c0 dk, c2 dk per component
 
   // a warp-uniform base and a 32-bit byte offset (cell_setup admits at most
   // 4e8 nodes: a component plane is below 2^32 bytes)
@@ -33,15 +34,15 @@ struct IO {
     return __ldg(reinterpret_cast<const T*>(reinterpret_cast<const char*>(p + plane) + o));
   }
   __device__ __forceinline__ T in(int d, unsigned o) const {
-    if (MODE == MM_PRE) return c0 * ld(dinv, d * nn, o) * ld(b, d * nn, o);
+    if (MODE == MM_PRE) return k0[d] * ld(dinv, 0, o) * ld(b, d * nn, o);
     return ld(x, d * nn, o);
   }
   __device__ __forceinline__ T rho(unsigned o) const { return ld(rp, 0, o); }
   __device__ __forceinline__ void fetch(Pre& p, unsigned o) const {
+    if (kStep) p.di = ld(dinv, 0, o);
 #pragma unroll
     for (int c = 0; c < NO; ++c) {
       if (kB) p.b[c] = ld(b, c * nn, o);
-      if (kStep) p.di[c] = ld(dinv, c * nn, o);
       // not through the read-only path: y may be xp (each node reads its own)
       if (kXp) p.xp[c] = *reinterpret_cast<const T*>(reinterpret_cast<const char*>(xp + c * nn) + o);
     }
@@ -59,9 +60,9 @@ struct IO {
         v = p.b[c] - acc[c];
       } else {
         const T x0 = own[c < NI ? c : 0];
-        v = x0 + c2 * p.di[c] * (p.b[c] - acc[c]);
+        v = x0 + k2[c] * p.di * (p.b[c] - acc[c]);
         if (MODE == MM_STEP) v += c1 * (x0 - p.xp[c]);
-        if (MODE == MM_STEP0) v += c1 * (x0 - c0 * p.di[c] * p.b[c]);
+        if (MODE == MM_STEP0) v += c1 * (x0 - k0[c] * p.di * p.b[c]);
         if (MODE == MM_PRE) v += c1 * x0;
       }
       *reinterpret_cast<T*>(reinterpret_cast<char*>(y + c * nn) + o) = v;
@@ -84,12 +85,14 @@ k_modal(const ModalArgs<T> a, const __grid_constant__ typename MatOf<KIND, T>::t
     io.dinv = a.dinv;
     io.rp = a.rho;
     io.nn = (i64)a.nx * a.ny * a.nz;
-    io.c0 = io.c1 = io.c2 = T(0);
     if (MODE >= MM_STEP) {
       io.c1 = a.c12[0];
-      io.c2 = a.c12[1];
+#pragma unroll
+      for (int c = 0; c < Shape<KIND>::NO; ++c) {
+        io.k2[c] = a.c12[1] * a.dk[c];
+        if (MODE == MM_STEP0 || MODE == MM_PRE) io.k0[c] = *a.c0 * a.dk[c];
+      }
     }
-    if (MODE == MM_STEP0 || MODE == MM_PRE) io.c0 = *a.c0;
     march<KIND, RY, PF, T>(K, io, a.nx, a.ny, a.nz, L);
   }
 }
