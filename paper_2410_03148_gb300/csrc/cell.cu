@@ -217,6 +217,8 @@ struct BlockMG {
   std::vector<T> cc_host;      // staging of the Chebyshev coefficients of all levels
   T* cc_dev = nullptr;
   unsigned int* lbits = nullptr;  // per-level lambda_max bounds (float bits)
+  double* dwork = nullptr;        // coarsest inverse on the device: workspace, element matrix
+  double* dk = nullptr;
 };
 
 template <typename T>
@@ -261,6 +263,7 @@ struct cell_handle {
   bool modal = false;            // mm2 material: operators in modal form
   ModalSet<float> m32;
   ModalSet<double> m64;
+  unsigned* dense_dev = nullptr;      // residuals of the two coarsest inverses (float bits)
   std::vector<void*> rho_lv, di_lv;   // per multigrid level (solver precision): element scales, inverse diagonals
   cell::ModalMat<cell::DF, 4, 4> mdf;
   Arena arena;
@@ -788,6 +791,11 @@ int alloc_mg_modal(cell_handle* h, BlockMG<T>& mg) {
   if (nd <= 3000) {
     CKS(h->arena.alloc(&Lc.dense, (size_t)nd * nd));
     Lc.ndense = (int)nd;
+    if (cell::dense_invert_ok((int)nd)) {
+      CKS(h->arena.alloc(&mg.dwork, cell::dense_invert_work((int)nd)));
+      CKS(h->arena.alloc(&mg.dk, R * R));
+      CK(cudaMemcpy(mg.dk, Lc.kb.data(), R * R * sizeof(double), cudaMemcpyHostToDevice));
+    }
   }
   // Chebyshev coefficients (the bounds do not depend on the design): (0, 1 / theta),
   // then (c1_k, c2_k)
@@ -811,6 +819,16 @@ cell::GridPair grid_pair(const Level<T>& F, const Level<T>& C) {
   return cell::GridPair{{F.nx, F.ny, F.nz}, {C.nx, C.ny, C.nz}};
 }
 
+// Coarsest inverse of one block: on the device up to its size limit, else on
+// the host (which waits for the stream).
+template <typename T, int NC>
+int start_inverse(cell_handle* h, BlockMG<T>& mg, int block) {
+  Level<T>& Lc = mg.lv.back();
+  if (!mg.dwork) return dense_inverse<T, NC>(h, mg);
+  cell::dense_invert<T>(Lc.rho, mg.dk, NC, Lc.nx, Lc.ny, Lc.nz, mg.dwork, Lc.dense, h->dense_dev + block, h->st);
+  return CELL_OK;
+}
+
 // Numerics of both hierarchies for the current rho: scales and diagonals of
 // every level, the coarsest inverses.
 template <typename T>
@@ -821,8 +839,18 @@ int fill_mg_modal(cell_handle* h) {
     if (l > 0) cell::mg_rho<T>(lv[l - 1].rho, static_cast<T*>(h->rho_lv[l]), grid_pair(lv[l - 1], lv[l]), h->st);
     cell::mg_dinv<T>(lv[l].rho, static_cast<T*>(h->di_lv[l]), lv[l].nx, lv[l].ny, lv[l].nz, h->st);
   }
-  CKS((dense_inverse<T, 3>(h, K.mgu)));
-  CKS((dense_inverse<T, 1>(h, K.mgp)));
+  CKS((start_inverse<T, 3>(h, K.mgu, 0)));
+  CKS((start_inverse<T, 1>(h, K.mgp, 1)));
+  return CELL_OK;
+}
+
+// After fill_mg_modal's launches have run: coarsest inverses that the device
+// could not form (an extreme contrast of rho) are formed on the host.
+template <typename T>
+int finish_mg_modal(cell_handle* h, const unsigned dev[2]) {
+  Krylov<T>& K = kry<T>(h);
+  if (K.mgu.dwork && cell::dense_invert_failed(dev[0])) CKS((dense_inverse<T, 3>(h, K.mgu)));
+  if (K.mgp.dwork && cell::dense_invert_failed(dev[1])) CKS((dense_inverse<T, 1>(h, K.mgp)));
   return CELL_OK;
 }
 
@@ -1041,7 +1069,6 @@ int setup_krylov(cell_handle* h) {
 
 template <typename T>
 int fill_krylov(cell_handle* h) {
-  if (h->modal) return fill_mg_modal<T>(h);
   Krylov<T>& K = kry<T>(h);
   CKS((fill_mg<T, 3>(h, K.mgu)));
   CKS((fill_mg<T, 1>(h, K.mgp)));
@@ -1222,11 +1249,16 @@ int load_design(cell_handle* h, const void* input) {
   }
   // rho_l = fp32(rho64 - rho32)
   cell::split_f64(h->rho64, h->rho_tmp, h->rho_l, nn, h->st);
+  cell::sum_reduce(h->rho64, nn, h->partial, h->nblk, h->red, h->st, 1);
+  const bool mixed = d->opt.precision == CELL_MIXED_FP32;
+  // mm2 materials: everything that follows is enqueued before the one wait
+  if (h->modal) CKS(mixed ? fill_mg_modal<float>(h) : fill_mg_modal<double>(h));
   double srho2 = 0.0;
   int nbad = 0;
-  cell::sum_reduce(h->rho64, nn, h->partial, h->nblk, h->red, h->st, 1);
+  unsigned dev[2] = {0, 0};
   CK(cudaMemcpyAsync(&srho2, h->red, sizeof(double), cudaMemcpyDeviceToHost, h->st));
   CK(cudaMemcpyAsync(&nbad, h->bad, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+  CK(cudaMemcpyAsync(dev, h->dense_dev, sizeof(dev), cudaMemcpyDeviceToHost, h->st));
   CK(cudaStreamSynchronize(h->st));
   if (nbad) {
     set_error("rho input has non-positive or non-finite values");
@@ -1240,8 +1272,8 @@ int load_design(cell_handle* h, const void* input) {
   // the whole-solve graph reads the floors from device memory (h->bfloor
   // outlives the copy)
   CK(cudaMemcpyAsync(h->bfloor_d, h->bfloor, sizeof(h->bfloor), cudaMemcpyHostToDevice, h->st));
-  if (d->opt.precision == CELL_MIXED_FP32) CKS(fill_krylov<float>(h));
-  else CKS(fill_krylov<double>(h));
+  if (h->modal) CKS(mixed ? finish_mg_modal<float>(h, dev) : finish_mg_modal<double>(h, dev));
+  else CKS(mixed ? fill_krylov<float>(h) : fill_krylov<double>(h));
   h->solved = false;
   CK(cudaGetLastError());
   return CELL_OK;
@@ -1322,6 +1354,8 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
   CKS(A.alloc(&h->rho_l, nn));
   CKS(A.alloc(&h->rho_tmp, nn));
   CKS(A.alloc(&h->bad, 1));
+  CKS(A.alloc(&h->dense_dev, 2));
+  CK(cudaMemsetAsync(h->dense_dev, 0, 2 * sizeof(unsigned), h->st));
   CKS(A.alloc(&h->dptrs, 1 + cell::kHilbertMaxCons));
   CKS(A.alloc(&h->bn2d, 9 * kNvMax));
   CKS(A.alloc(&h->relres_d, 9));

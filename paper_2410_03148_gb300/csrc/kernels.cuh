@@ -264,6 +264,17 @@ template <typename T> void mg_dinv(const T* rho, T* dinv, int nx, int ny, int nz
 template <typename T, int NC> void mg_scale(const T* b, i64 bs, T* x, i64 xs, const T* dinv, const T* dk, const T* c0,
                                             i64 nn, int nrhs, const int* active, cudaStream_t s);
 
+// Coarsest inverse on the device (dense.cu), n = nc nx ny nz <= the limit of
+// dense_invert_ok: out = (sum_e rho_e P_e^T K P_e + regularisation)^-1; K:
+// device, (8 nc)^2 FP64; work: dense_invert_work(n) doubles; *dev receives the
+// float bits of the residual before the last correction, to be judged with
+// dense_invert_failed.
+bool dense_invert_ok(int n);
+size_t dense_invert_work(int n);
+bool dense_invert_failed(unsigned dev_bits);
+template <typename T> void dense_invert(const T* rho, const double* K, int nc, int nx, int ny, int nz, double* work,
+                                        T* out, unsigned* dev, cudaStream_t s);
+
 // ---- multigrid helpers (mg.cu) ----------------------------------------------
 // r = b, d = c2 Dinv b with c2 read from device memory (*c2p)
 template <typename T, int NC> void cheb_init(const T* b, i64 bs, T* r, i64 rs, T* d, i64 ds,
