@@ -349,22 +349,28 @@ template <typename T> const ModalSet<T>& modal_of(const cell_handle* h);
 template <> const ModalSet<float>& modal_of<float>(const cell_handle* h) { return h->m32; }
 template <> const ModalSet<double>& modal_of<double>(const cell_handle* h) { return h->m64; }
 
-// Blocks of one, two and three differences of rows o0 .. o0 + NO - 1 and
-// columns 0 .. NI - 1 of a modal matrix over nc components.
+// Rows of output components o0 .. o0 + NO - 1 and input components 0 .. NI - 1
+// of a modal matrix over nc components (ModalMat's order).
 template <int NO, int NI, typename V, typename F>
 void fill_modal(const double* Km, int nc, int o0, cell::ModalMat<V, NO, NI>& M, F&& conv) {
   const int R = 8 * nc;
-  auto at = [&](int m, int c, int n, int d) { return conv(Km[(m * nc + o0 + c) * R + n * nc + d]); };
-  for (int c = 0; c < NO; ++c)
-    for (int d = 0; d < NI; ++d) {
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-          const int k = (i * NO + c) * 3 * NI + j * NI + d;
-          M.c[k] = at(1 << i, c, 1 << j, d);
-          M.q[k] = at(7 ^ (1 << i), c, 7 ^ (1 << j), d);
-        }
-      M.t[c * NI + d] = at(7, c, 7, d);
+  auto row = [&](int c, int m, int cls) {
+    cell::ModalRow<V> r{};
+    int n = 0;
+    for (int j = 0; j < (cls == 2 ? 1 : 3); ++j)
+      for (int d = 0; d < NI; ++d) {
+        const int mode = cls == 0 ? 1 << j : (cls == 1 ? 7 ^ (1 << j) : 7);
+        if (cell::modal_couples(o0 + c, m, d, mode)) r.v[n++] = conv(Km[(m * nc + o0 + c) * R + mode * nc + d]);
+      }
+    return r;
+  };
+  for (int c = 0; c < NO; ++c) {
+    for (int i = 0; i < 3; ++i) {
+      M.c[i * NO + c] = row(c, 1 << i, 0);
+      M.q[i * NO + c] = row(c, 7 ^ (1 << i), 1);
     }
+    M.t[c] = row(c, 7, 2);
+  }
 }
 
 template <typename T>

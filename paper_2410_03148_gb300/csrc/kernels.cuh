@@ -97,6 +97,16 @@ struct ApplyArgs {
 };
 
 // ---- modal element operators (modal.cuh, modal_f32.cu, modal_f64.cu) -----------
+struct DF {         // unevaluated pair h + l
+  float h, l;
+};
+// Mirror parity of dof (component c, mode m): a displacement component and
+// its own axis' difference flip together, the potential with z.  An mm2
+// material couples only dofs of equal parity.
+__host__ __device__ constexpr int modal_parity(int c, int m) { return m ^ (c == 0 ? 1 : (c == 1 ? 2 : 4)); }
+__host__ __device__ constexpr bool modal_couples(int c, int m, int c2, int m2) {
+  return modal_parity(c, m) == modal_parity(c2, m2);
+}
 enum ModalKind { MK_FULL = 0, MK_UU = 1, MK_PU = 2, MK_SS = 3 };   // Ahat, A, B, Sbar
 enum ModalMode {
   MM_APPLY = 0,   // y = A x
@@ -112,20 +122,23 @@ enum ModalMode {
   MM_PRE = 5,     // the same with x_k = c0 D^-1 b (not stored) and x_{k-1} = 0
   MM_POST = 6     // y = x + c2 D^-1 (b - A x)
 };
-// Modal element matrix K^ (modal.cuh), blocks of one (c), two (q) and three
-// (t) differences: c[(i NO + c) 3 NI + j NI + d] couples output component c of
-// the mode "difference along i" with input component d of "difference along
-// j"; q likewise for the modes "difference along all axes but i".
+// Modal element matrix K^ (modal.cuh): a row of (at most) four entries per
+// output dof, the coupled input dofs in order.  c[i NO + o]: mode "difference
+// along i" of output component o, coupled with the modes "difference along j"
+// of the input components d in the order j NI + d; q: likewise the modes
+// "difference along all axes but i"; t[o]: the mode of three differences.
+// Rows are fetched as one 16- or 32-byte constant load.
+template <typename T>
+struct alignas(4 * sizeof(T)) ModalRow {
+  T v[4];
+};
 template <typename T, int NO, int NI>
 struct ModalMat {
-  T c[9 * NO * NI], q[9 * NO * NI], t[NO * NI];
+  ModalRow<T> c[3 * NO], q[3 * NO], t[NO];
 };
 template <typename T>
-struct ModalSch {   // diagonal of Sbar's modal matrix, modes 1..7
+struct alignas(4 * sizeof(T)) ModalSch {   // diagonal of Sbar's modal matrix, modes 1..7
   T s[8];
-};
-struct DF {         // unevaluated pair h + l
-  float h, l;
 };
 // One operator launch.  Vectors as in ApplyArgs: value(load q, comp c, node n)
 // = p[q * stride + c * nn + n].

@@ -35,11 +35,6 @@ constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
 constexpr int kOut = 30;   // output columns of a warp
 
-// Mirror parity of dof (component c, mode m): a displacement component and
-// its own axis' difference flip together; the potential flips with z.
-__host__ __device__ constexpr int parity(int c, int m) { return m ^ (c == 0 ? 1 : (c == 1 ? 2 : 4)); }
-__host__ __device__ constexpr bool couples(int c, int m, int c2, int m2) { return parity(c, m) == parity(c2, m2); }
-
 // ---- arithmetic -------------------------------------------------------------
 // Value types: float, double, and DF, an unevaluated pair h + l of floats with
 // error-free products and sums of the leading parts (about 2^-46).
@@ -107,24 +102,17 @@ __device__ __forceinline__ Pair<float> pmul(float k, const Pair<float>& a) {
 }
 
 // ---- element contraction ------------------------------------------------------
-// f[c][m] = sum K^[(c,m)][(d,n)] u[d][n] within the classes of one, two and
-// three differences.  CO = component of the first output row.
-//
-// first input dof (j NI + d, from 0) that row (c, mode) of a class couples
-// with; mode of axis j: 1 << j, or 7 without it
+// Coupled input dofs before the k-th (k = j NI + d) in the row of output dof
+// (c, mode); two: modes of two differences (7 without axis j).
 template <int NI>
-__host__ __device__ constexpr int first_of(int c, int m, bool two) {
-  for (int k = 0; k < 3 * NI; ++k)
-    if (couples(c, m, k % NI, two ? 7 ^ (1 << (k / NI)) : 1 << (k / NI))) return k;
-  return -1;
-}
-template <int NI>
-__host__ __device__ constexpr int first_of3(int c) {
-  for (int d = 0; d < NI; ++d)
-    if (couples(c, 7, d, 7)) return d;
-  return -1;
+__host__ __device__ constexpr int before(int c, int m, int k, bool two) {
+  int n = 0;
+  for (int q = 0; q < k; ++q) n += modal_couples(c, m, q % NI, two ? 7 ^ (1 << (q / NI)) : 1 << (q / NI)) ? 1 : 0;
+  return n;
 }
 
+// f[c][m] = sum K^[(c,m)][(d,n)] u[d][n] within the classes of one, two and
+// three differences.  CO = component of the first output row.
 template <int NO, int NI, int CO, typename V>
 __device__ __forceinline__ void force(const ModalMat<V, NO, NI>& K, const V (&u)[NI][8], V (&f)[NO][8]) {
 #pragma unroll
@@ -132,23 +120,32 @@ __device__ __forceinline__ void force(const ModalMat<V, NO, NI>& K, const V (&u)
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const int m1 = 1 << i, m2 = 7 ^ m1;
+      const ModalRow<V> k1 = K.c[i * NO + c], k2 = K.q[i * NO + c];
       V f1 = V{}, f2 = V{};
 #pragma unroll
       for (int k = 0; k < 3 * NI; ++k) {
-        const int j = k / NI, d = k % NI, n1 = 1 << j, n2 = 7 ^ n1, at = (i * NO + c) * 3 * NI + k;
-        if (couples(CO + c, m1, d, n1))
-          f1 = k == first_of<NI>(CO + c, m1, false) ? vmul(K.c[at], u[d][n1]) : vfma(K.c[at], u[d][n1], f1);
-        if (couples(CO + c, m2, d, n2))
-          f2 = k == first_of<NI>(CO + c, m2, true) ? vmul(K.q[at], u[d][n2]) : vfma(K.q[at], u[d][n2], f2);
+        const int j = k / NI, d = k % NI, n1 = 1 << j, n2 = 7 ^ n1;
+        if (modal_couples(CO + c, m1, d, n1)) {
+          const int at = before<NI>(CO + c, m1, k, false);
+          f1 = at == 0 ? vmul(k1.v[at], u[d][n1]) : vfma(k1.v[at], u[d][n1], f1);
+        }
+        if (modal_couples(CO + c, m2, d, n2)) {
+          const int at = before<NI>(CO + c, m2, k, true);
+          f2 = at == 0 ? vmul(k2.v[at], u[d][n2]) : vfma(k2.v[at], u[d][n2], f2);
+        }
       }
       f[c][m1] = f1;
       f[c][m2] = f2;
     }
+    const ModalRow<V> k3 = K.t[c];
     V f3 = V{};
+    int at = 0;
 #pragma unroll
     for (int d = 0; d < NI; ++d)
-      if (couples(CO + c, 7, d, 7))
-        f3 = d == first_of3<NI>(CO + c) ? vmul(K.t[c * NI + d], u[d][7]) : vfma(K.t[c * NI + d], u[d][7], f3);
+      if (modal_couples(CO + c, 7, d, 7)) {
+        f3 = at == 0 ? vmul(k3.v[at], u[d][7]) : vfma(k3.v[at], u[d][7], f3);
+        ++at;
+      }
     f[c][7] = f3;
   }
 }
@@ -204,8 +201,8 @@ __device__ __forceinline__ void element(const typename MatOf<KIND, V>::type& K, 
 }
 
 // ---- the march ------------------------------------------------------------------
-// IO supplies the inputs and takes the outputs of one load (offsets in bytes
-// from the start of a component plane):
+// IO supplies the inputs and takes the outputs of one load (offsets from the
+// start of a component plane):
 //   V    in(d, offset)          input component d at a node
 //   V    rho(offset)            element scale
 //   void fetch(pre, offset)     operands of a node's output
@@ -215,7 +212,6 @@ template <int KIND, int RY, bool PF, typename V, typename IO>
 __device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, const IO& io, int nx, int ny, int nz,
                                       int L) {
   constexpr int NI = Shape<KIND>::NI, NO = Shape<KIND>::NO;
-  constexpr unsigned SZ = IO::kBytes;
   const int lane = threadIdx.x & 31;
   const int rl = nx + 2;
   const int strips = (ny + RY - 1) / RY;
@@ -233,36 +229,28 @@ __device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, co
   bool ok[RY];
 #pragma unroll
   for (int r = 0; r < RY + 2; ++r) {
-    int j = j0 - 1 + r;
-    j = j < 0 ? j + ny : j % ny;
-    ro[r] = (unsigned)(j * nx + i) * SZ;
+    int j = j0 - 1 + r;   // at most ny + RY - 1: two subtractions wrap it (RY <= 4, ny >= 2)
+    j = j < 0 ? j + ny : j;
+    j = j >= ny ? j - ny : j;
+    j = j >= ny ? j - ny : j;
+    ro[r] = (unsigned)(j * nx + i);
   }
 #pragma unroll
   for (int r = 0; r < RY; ++r) ok[r] = vx && j0 + r < ny;
-  const unsigned nxy = (unsigned)(nx * ny) * SZ;
+  const unsigned nxy = (unsigned)(nx * ny);
   const int z0 = blockIdx.z * L;
   const int Lc = min(L, nz - z0);
   Pair<V> ps[RY + 2][NI];   // x sums and differences of the plane before
   V own[RY][NI];            // its values on the strip's own rows
   Pair<V> carry[RY][NO];    // contributions of the layer below to the plane before
   unsigned zp = (unsigned)(z0 == 0 ? nz - 1 : z0 - 1) * nxy;   // the plane before
+  unsigned zc = (unsigned)z0 * nxy;   // the plane above the layer
+  // the loads of the first two planes are in flight together
+  V v0[RY + 2][NI], vn[PF ? RY + 2 : 1][NI], rn[PF ? RY + 1 : 1];
 #pragma unroll
   for (int r = 0; r < RY + 2; ++r)
 #pragma unroll
-    for (int d = 0; d < NI; ++d) {
-      const V v = io.in(d, zp + ro[r]);
-      const V w = vdown(v);
-      ps[r][d] = mk<V>(vadd(w, v), vsub(w, v));
-    }
-#pragma unroll
-  for (int r = 0; r < RY; ++r) {
-#pragma unroll
-    for (int c = 0; c < NO; ++c) carry[r][c] = mk<V>(V{}, V{});
-#pragma unroll
-    for (int d = 0; d < NI; ++d) own[r][d] = V{};
-  }
-  unsigned zc = (unsigned)z0 * nxy;   // the plane above the layer
-  V vn[PF ? RY + 2 : 1][NI], rn[PF ? RY + 1 : 1];
+    for (int d = 0; d < NI; ++d) v0[r][d] = io.in(d, zp + ro[r]);
   if (PF) {
 #pragma unroll
     for (int r = 0; r < RY + 2; ++r)
@@ -270,6 +258,20 @@ __device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, co
       for (int d = 0; d < NI; ++d) vn[PF ? r : 0][d] = io.in(d, zc + ro[r]);
 #pragma unroll
     for (int r = 0; r < RY + 1; ++r) rn[PF ? r : 0] = io.rho(zp + ro[r]);
+  }
+#pragma unroll
+  for (int r = 0; r < RY + 2; ++r)
+#pragma unroll
+    for (int d = 0; d < NI; ++d) {
+      const V w = vdown(v0[r][d]);
+      ps[r][d] = mk<V>(vadd(w, v0[r][d]), vsub(w, v0[r][d]));
+    }
+#pragma unroll
+  for (int r = 0; r < RY; ++r) {
+#pragma unroll
+    for (int c = 0; c < NO; ++c) carry[r][c] = mk<V>(V{}, V{});
+#pragma unroll
+    for (int d = 0; d < NI; ++d) own[r][d] = V{};
   }
 #pragma unroll 1
   for (int t = 0; t <= Lc; ++t) {

@@ -6,7 +6,6 @@ namespace cell {
 namespace {
 
 struct DfIO {
-  static constexpr unsigned kBytes = 4;
   struct Pre {
     double b[4];
   };
@@ -15,20 +14,20 @@ struct DfIO {
   double* r;
   i64 nn;
   static __device__ __forceinline__ float ld(const float* p, i64 plane, unsigned o) {
-    return __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(p + plane) + o));
+    return __ldg(p + plane + o);
   }
   __device__ __forceinline__ DF in(int d, unsigned o) const { return {ld(xh, d * nn, o), ld(xl, d * nn, o)}; }
   __device__ __forceinline__ DF rho(unsigned o) const { return {ld(rh, 0, o), ld(rl, 0, o)}; }
   __device__ __forceinline__ void fetch(Pre& p, unsigned o) const {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) p.b[c] = b ? __ldg(b + c * nn + (o >> 2)) : 0.0;
+    for (int c = 0; c < 4; ++c) p.b[c] = b ? __ldg(b + c * nn + o) : 0.0;
   }
   __device__ __forceinline__ void out(unsigned o, DF (&acc)[4], const DF (&)[4], const Pre& p) const {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       double v = (double)acc[c].h + (double)acc[c].l;
       if (c == 3) v = -v;
-      r[c * nn + (o >> 2)] = b ? p.b[c] - v : v;
+      r[c * nn + o] = b ? p.b[c] - v : v;
     }
   }
 };

@@ -27,12 +27,7 @@ struct IO {
   T c1;
   T k0[3], k2[3];   // c0 dk, c2 dk per component
 
-  // a warp-uniform base and a 32-bit byte offset (cell_setup admits at most
-  // 4e8 nodes: a component plane is below 2^32 bytes)
-  static constexpr unsigned kBytes = sizeof(T);
-  __device__ __forceinline__ static T ld(const T* p, i64 plane, unsigned o) {
-    return __ldg(reinterpret_cast<const T*>(reinterpret_cast<const char*>(p + plane) + o));
-  }
+  __device__ __forceinline__ static T ld(const T* p, i64 plane, unsigned o) { return __ldg(p + plane + o); }
   __device__ __forceinline__ T in(int d, unsigned o) const {
     if (MODE == MM_PRE) return k0[d] * ld(dinv, 0, o) * ld(b, d * nn, o);
     return ld(x, d * nn, o);
@@ -44,7 +39,7 @@ struct IO {
     for (int c = 0; c < NO; ++c) {
       if (kB) p.b[c] = ld(b, c * nn, o);
       // not through the read-only path: y may be xp (each node reads its own)
-      if (kXp) p.xp[c] = *reinterpret_cast<const T*>(reinterpret_cast<const char*>(xp + c * nn) + o);
+      if (kXp) p.xp[c] = xp[c * nn + o];
     }
   }
   __device__ __forceinline__ void out(unsigned o, T (&acc)[NO], const T (&own)[NI], const Pre& p) const {
@@ -65,7 +60,7 @@ struct IO {
         if (MODE == MM_STEP0) v += c1 * (x0 - k0[c] * p.di * p.b[c]);
         if (MODE == MM_PRE) v += c1 * x0;
       }
-      *reinterpret_cast<T*>(reinterpret_cast<char*>(y + c * nn) + o) = v;
+      y[c * nn + o] = v;
     }
   }
 };
@@ -76,7 +71,8 @@ k_modal(const ModalArgs<T> a, const __grid_constant__ typename MatOf<KIND, T>::t
   const int r1 = min(a.nrhs, ((int)blockIdx.y + 1) * a.rg);
 #pragma unroll 1
   for (int r = blockIdx.y * a.rg; r < r1; ++r) {
-    if (a.active && !a.active[r]) continue;
+    // a vote, so that the branch (and every address below) is warp-uniform
+    if (a.active && !__any_sync(0xffffffffu, a.active[r])) continue;
     IO<KIND, MODE, T> io;
     io.x = a.x + r * a.xs;
     io.y = a.y + r * a.ys;
