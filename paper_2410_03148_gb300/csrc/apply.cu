@@ -638,36 +638,6 @@ k_resid_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs,
   }
 }
 
-__global__ void k_axpy_split_f(double* __restrict__ x, float* __restrict__ xh, float* __restrict__ xl,
-                               i64 xs, const float* __restrict__ d, i64 ds, i64 len,
-                               const double* __restrict__ sc, const int* active) {
-  const int q = blockIdx.y;
-  if (active && !active[q]) return;
-  const double f = sc[q];
-  for (i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x; k < len; k += (i64)gridDim.x * blockDim.x) {
-    const double v = x[q * xs + k] + f * (double)d[q * ds + k];
-    x[q * xs + k] = v;
-    const float h = (float)v;
-    xh[q * xs + k] = h;
-    xl[q * xs + k] = (float)(v - (double)h);
-  }
-}
-
-__global__ void k_axpy_split_d(double* __restrict__ x, float* __restrict__ xh, float* __restrict__ xl,
-                               i64 xs, const double* __restrict__ d, i64 ds, i64 len,
-                               const double* __restrict__ sc, const int* active) {
-  const int q = blockIdx.y;
-  if (active && !active[q]) return;
-  const double f = sc[q];
-  for (i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x; k < len; k += (i64)gridDim.x * blockDim.x) {
-    const double v = x[q * xs + k] + f * d[q * ds + k];
-    x[q * xs + k] = v;
-    const float h = (float)v;
-    xh[q * xs + k] = h;
-    xl[q * xs + k] = (float)(v - (double)h);
-  }
-}
-
 template <typename T>
 inline dim3 grid_for(const ApplyArgs<T>& a, int nrhs) {
   const int plane = a.nx * a.ny;
@@ -874,21 +844,6 @@ void split_f64(const double* x, float* xh, float* xl, i64 n, cudaStream_t s) {
   if (blocks > 8192) blocks = 8192;
   note_launch(), k_split<<<(unsigned)blocks, 256, 0, s>>>(x, xh, xl, n);
 }
-
-template <typename T>
-void axpy_split(double* x, float* xh, float* xl, i64 xs, const T* d, i64 ds, i64 len,
-                const double* sc, int nrhs, const int* active, cudaStream_t s) {
-  i64 blocks = (len + 255) / 256;
-  if (blocks > 4096) blocks = 4096;
-  if constexpr (sizeof(T) == 4)
-    note_launch(), k_axpy_split_f<<<dim3((unsigned)blocks, nrhs), 256, 0, s>>>(x, xh, xl, xs, d, ds, len, sc, active);
-  else
-    note_launch(), k_axpy_split_d<<<dim3((unsigned)blocks, nrhs), 256, 0, s>>>(x, xh, xl, xs, d, ds, len, sc, active);
-}
-template void axpy_split<float>(double*, float*, float*, i64, const float*, i64, i64, const double*,
-                                int, const int*, cudaStream_t);
-template void axpy_split<double>(double*, float*, float*, i64, const double*, i64, i64,
-                                 const double*, int, const int*, cudaStream_t);
 
 // ---- constant-bank slot manager ---------------------------------------------
 namespace {

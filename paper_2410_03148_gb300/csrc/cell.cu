@@ -227,7 +227,6 @@ struct Krylov {
   i64 len = 0;
   T* V = nullptr;        // (m+1) x 9 x len
   T* Z = nullptr;        // m x 9 x len: preconditioned directions z_j = P^-1 v_j (flexible GMRES)
-  T* u = nullptr;        // 9 x len
   T* tphi = nullptr;     // 9 x nn (Schur block right-hand side)
   T* ru = nullptr;       // 9 x 3nn (extra elastic V-cycles)
   T* eu = nullptr;
@@ -291,10 +290,12 @@ struct cell_handle {
   // right-hand sides or residuals below 1e-13 of it are rounding noise
   double bfloor[9];
   // Krylov-scalar state (FP64, device)
-  double *H = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr, *hcol = nullptr, *hnorm = nullptr;
+  double *H = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr, *hcol = nullptr;
+  double *gram = nullptr, *nu2 = nullptr, *coef = nullptr, *gs_partial = nullptr;   // Gram-Schmidt (gs.cu)
+  int gs_nblk = 1;
+  int* ticket = nullptr;
   double *resid = nullptr, *invscale = nullptr, *tolabs = nullptr, *ybuf = nullptr, *beta2 = nullptr;
-  double* ones = nullptr;
-  int *active = nullptr, *kcount = nullptr, *want = nullptr, *ranmask = nullptr, *reorth = nullptr;
+  int *active = nullptr, *kcount = nullptr, *want = nullptr, *ranmask = nullptr;
   Krylov<float> kf;
   Krylov<double> kd;
   bool solved = false;
@@ -1047,7 +1048,6 @@ int setup_krylov(cell_handle* h) {
   for (int i = 0; i < 64; ++i) K.S0.k[i] = (T)h->S0[i];
   CKS(h->arena.alloc(&K.V, (size_t)(K.m + 1) * 9 * K.len));
   CKS(h->arena.alloc(&K.Z, (size_t)K.m * 9 * K.len));
-  CKS(h->arena.alloc(&K.u, (size_t)9 * K.len));
   CKS(h->arena.alloc(&K.tphi, (size_t)9 * h->nn));
   if (o.vcycles_u > 1) {
     CKS(h->arena.alloc(&K.ru, (size_t)27 * h->nn));
@@ -1083,41 +1083,29 @@ int fill_krylov(cell_handle* h) {
 
 // One Arnoldi step j of the batched GMRES (all kernels, no host sync):
 // z = P^-1 v_j, w = Ahat z, Gram-Schmidt against v_0..v_j, Givens update,
-// normalisation.  Launches go to h->st (the capture stream while captured).
+// normalisation.  Launches go to h->st (the capture stream while captured);
+// inside a solve graph the step sets the condition of the next one.
 template <typename T>
-void iteration(cell_handle* h, int j) {
+void iteration(cell_handle* h, int j, cudaGraphConditionalHandle next = 0, bool set_next = false) {
   Krylov<T>& K = kry<T>(h);
-  const int m = K.m;
   const i64 len = K.len;
   const i64 vstride = 9 * len;
   cudaStream_t s = h->st;
-  const int nblk = h->nblk;
   T* vj = K.V + (i64)j * vstride;
   T* w = K.V + (i64)(j + 1) * vstride;
   T* zj = K.Z + (i64)j * vstride;
   precond<T>(h, vj, zj, h->active);
   apply_full_T<T>(h, zj, len, w, len, nullptr, 0, h->active, 9);
-  // Classical Gram-Schmidt with selective reorthogonalisation: one pass of
-  // dots (w is V_{j+1}, so the same pass also gives |w|^2); one pass that
-  // updates w and, from the same basis reads, forms the second pass's dots
-  // and the new norm; a second update only for loads whose norm dropped
-  // below 1/sqrt(2) of its value before the first (three basis passes).
   const int ipk = h->prof.begin(s, CELL_PROF_KRYLOV);
-  cell::multidot<T>(K.V, vstride, len, j + 2, w, len, len, h->partial, nblk, kNvMax, 9, h->active, s);
-  cell::reduce_partials(h->partial, nblk, j + 2, kNvMax, h->hcol, 0, 9, h->active, s);
-  // first update fused with the second pass's dots and the new norm
-  cell::update_dots<T>(K.V, vstride, len, j + 1, h->hcol, kNvMax, w, len, len, h->partial, nblk, 9, h->active, s);
-  cell::reduce_partials(h->partial + (j + 1), nblk, 1, kNvMax, h->hnorm, 0, 9, h->active, s);
-  cell::reorth_flag(h->hcol, h->hnorm, j, h->active, h->reorth, 9, s);
-  cell::reduce_partials(h->partial, nblk, j + 1, kNvMax, h->ybuf, 0, 9, h->reorth, s);
-  cell::update<T>(K.V, vstride, len, j + 1, h->ybuf, kNvMax, w, len, len, 2, h->partial, nblk, 9, h->reorth, s);
-  cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->hnorm, 0, 9, h->reorth, s);
-  // hcol += second-pass coefficients (a one-block "reduction" of ybuf)
-  cell::reduce_partials(h->ybuf, 1, j + 1, kNvMax, h->hcol, 1, 9, h->reorth, s);
+  cell::GsArgs<T> a{};
+  a.V = K.V; a.vstride = vstride; a.len = len;
+  a.partial = h->gs_partial; a.nblk = h->gs_nblk;
+  a.gram = h->gram; a.nu2 = h->nu2; a.coef = h->coef; a.hcol = h->hcol;
+  a.H = h->H; a.cs = h->cs; a.sn = h->sn; a.g = h->g; a.resid = h->resid; a.tolabs = h->tolabs;
+  a.active = h->active; a.kcount = h->kcount; a.ticket = h->ticket;
+  a.m = K.m; a.nrhs = 9;
+  cell::gs_step<T>(a, j, next, set_next, s);
   h->prof.end(CELL_PROF_KRYLOV, ipk, s);
-  cell::givens_step(h->H, h->cs, h->sn, h->g, h->hcol, h->hnorm, j, m, h->active, h->resid,
-                    h->tolabs, h->invscale, h->kcount, 9, s);
-  cell::scale_vec<T>(w, len, len, h->invscale, 9, s);
 }
 
 // One restarted GMRES cycle (<= m iterations) on Ahat d = r64 for the loads
@@ -1134,13 +1122,12 @@ int gmres_cycle(cell_handle* h, const double* tolabs_host, int* iters) {
   cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, h->want, s);
   cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->beta2, 0, 9, h->want, s);
   CK(cudaMemcpyAsync(h->tolabs, tolabs_host, 9 * sizeof(double), cudaMemcpyHostToDevice, s));
-  cell::start_cycle(h->beta2, h->g, m, h->active, h->want, h->resid, h->invscale, h->tolabs, h->kcount, 9, s);
+  cell::start_cycle(h->beta2, h->g, h->nu2, m, h->active, h->want, h->resid, h->invscale, h->tolabs, h->kcount, 9, s);
   CK(cudaMemcpyAsync(h->ranmask, h->active, 9 * sizeof(int), cudaMemcpyDeviceToDevice, s));
   if constexpr (sizeof(T) == 4) {
     cell::to_f32_scaled(h->r64, len, reinterpret_cast<float*>(K.V), len, len, h->invscale, 9, h->ranmask, s);
   } else {
-    CK(cudaMemcpyAsync(K.V, h->r64, 9 * len * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    cell::scale_vec<T>(K.V, len, len, h->invscale, 9, s);
+    cell::copy_scale_f64(h->r64, reinterpret_cast<double*>(K.V), len, h->invscale, 9, h->ranmask, s);
   }
   int ran[9];
   CK(cudaMemcpyAsync(ran, h->ranmask, sizeof(ran), cudaMemcpyDeviceToHost, s));
@@ -1199,15 +1186,11 @@ int gmres_cycle(cell_handle* h, const double* tolabs_host, int* iters) {
     nunits = nact;
   }
   h->prof.cur_units = nran;
-  cell::backsolve(h->H, h->g, h->kcount, m, h->ybuf, 9, h->ranmask, s);
+  cell::backsolve(h->H, h->g, h->nu2, h->kcount, m, h->ybuf, 9, h->ranmask, s);
 
   // flexible GMRES: d = Z y with the stored preconditioned directions, so the
   // preconditioner may vary between iterations (reduced-precision smoothers)
-  cell::lincomb<T>(K.Z, vstride, len, h->ybuf, h->kcount, kNvMax, K.u, len, len, 9, h->ranmask, s);
-  if constexpr (sizeof(T) == 4)
-    cell::axpy_split<T>(h->x64, h->xh, h->xl, len, K.u, len, len, h->ones, 9, h->ranmask, s);
-  else
-    cell::axpy_f64<T>(h->x64, len, K.u, len, len, h->ones, 9, h->ranmask, s);
+  cell::gs_solution<T>(K.Z, vstride, len, h->ybuf, h->kcount, h->x64, h->xh, h->xl, 9, h->ranmask, s);
   int kc[9];
   CK(cudaMemcpyAsync(kc, h->kcount, sizeof(kc), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
@@ -1414,22 +1397,22 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
   CKS(A.alloc(&h->sn, 9 * m));
   CKS(A.alloc(&h->g, 9 * (m + 1)));
   CKS(A.alloc(&h->hcol, 9 * kNvMax));
-  CKS(A.alloc(&h->hnorm, 9 * kNvMax));
+  CKS(A.alloc(&h->gram, 9 * kNvMax * kNvMax));
+  CKS(A.alloc(&h->nu2, 9 * kNvMax));
+  CKS(A.alloc(&h->coef, 9 * (kNvMax + 1)));
+  h->gs_nblk = cell::gs_blocks(len);
+  CKS(A.alloc(&h->gs_partial, (size_t)9 * kNvMax * h->gs_nblk));
+  CKS(A.alloc(&h->ticket, 1));
+  CK(cudaMemsetAsync(h->ticket, 0, sizeof(int), h->st));
   CKS(A.alloc(&h->ybuf, 9 * kNvMax));
   CKS(A.alloc(&h->beta2, 9 * kNvMax));
   CKS(A.alloc(&h->resid, 9));
   CKS(A.alloc(&h->invscale, 9));
   CKS(A.alloc(&h->tolabs, 9));
-  CKS(A.alloc(&h->ones, 9));
-  {
-    const double one9[9] = {1, 1, 1, 1, 1, 1, 1, 1, 1};
-    CK(cudaMemcpyAsync(h->ones, one9, sizeof(one9), cudaMemcpyHostToDevice, h->st));
-  }
   CKS(A.alloc(&h->active, 9));
   CKS(A.alloc(&h->kcount, 9));
   CKS(A.alloc(&h->want, 9));
   CKS(A.alloc(&h->ranmask, 9));
-  CKS(A.alloc(&h->reorth, 9));
   CK(cudaMemsetAsync(h->x64, 0, 9 * len * sizeof(double), h->st));
   if (d->opt.precision == CELL_MIXED_FP32) {
     float k0f[1024], s0f[64];
@@ -1549,10 +1532,8 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
       cell::multidot<double>(h->b64, 0, len, 1, h->b64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
       cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->bn2d, 0, 9, nullptr, s);
       cudaMemcpyAsync(h->r64, h->b64, 9 * len * sizeof(double), cudaMemcpyDeviceToDevice, s);
-      cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
-      cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->red, 0, 9, nullptr, s);
       cell::ctl_reset(h->ctl_d, h->iters_d, s);
-      cell::refine_ctl(h->bn2d, h->red, h->bfloor_d, P, h->want, h->tolabs, h->relres_d, h->iters_d, h->ctl_d, wh, s);
+      cell::refine_ctl(h->bn2d, h->bn2d, h->bfloor_d, P, h->want, h->tolabs, h->relres_d, h->iters_d, h->ctl_d, wh, s);
       cudaError_t e1 = add_conditional(h, wh, cudaGraphCondTypeWhile, &wbody);
       if (e1 != cudaSuccess) return e1;
       const long long nb = cell::g_launches.load();
@@ -1573,7 +1554,7 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
       cudaStream_t s = h->st;
       cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, h->want, s);
       cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->beta2, 0, 9, h->want, s);
-      cell::start_cycle(h->beta2, h->g, m, h->active, h->want, h->resid, h->invscale, h->tolabs, h->kcount, 9, s);
+      cell::start_cycle(h->beta2, h->g, h->nu2, m, h->active, h->want, h->resid, h->invscale, h->tolabs, h->kcount, 9, s);
       cell::cycle_handles(h->active, h->ranmask, IH, s);
       if constexpr (sizeof(T) == 4)
         cell::to_f32_scaled(h->r64, len, reinterpret_cast<float*>(K.V), len, len, h->invscale, 9, h->ranmask, s);
@@ -1584,12 +1565,8 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
         if (e1 != cudaSuccess) return e1;
       }
       const long long nb = cell::g_launches.load();
-      cell::backsolve(h->H, h->g, h->kcount, m, h->ybuf, 9, h->ranmask, s);
-      cell::lincomb<T>(K.Z, 9 * len, len, h->ybuf, h->kcount, kNvMax, K.u, len, len, 9, h->ranmask, s);
-      if constexpr (sizeof(T) == 4)
-        cell::axpy_split<T>(h->x64, h->xh, h->xl, len, K.u, len, len, h->ones, 9, h->ranmask, s);
-      else
-        cell::axpy_f64<T>(h->x64, len, K.u, len, len, h->ones, 9, h->ranmask, s);
+      cell::backsolve(h->H, h->g, h->nu2, h->kcount, m, h->ybuf, 9, h->ranmask, s);
+      cell::gs_solution<T>(K.Z, 9 * len, len, h->ybuf, h->kcount, h->x64, h->xh, h->xl, 9, h->ranmask, s);
       cell::accum_iters(h->iters_d, h->kcount, h->ranmask, h->ctl_d, s);
       if constexpr (sizeof(T) == 4)
         residual_df(h, h->b64, h->r64, 9);
@@ -1605,8 +1582,8 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
   long long n_it = 0, n_it0 = 0;
   for (int j = 0; j < m && e == cudaSuccess; ++j) {
     e = capture_into(h, ifbody[j], [&]() -> cudaError_t {
-      iteration<T>(h, j);
-      if (j + 1 < m) cell::next_step(h->active, IH.h[j + 1], h->st);
+      if (j + 1 < m) iteration<T>(h, j, IH.h[j + 1], true);
+      else iteration<T>(h, j);
       return cudaGetLastError();
     }, &n_it);
     if (j == 0) n_it0 = n_it;
@@ -1618,7 +1595,7 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
   h->seg_epi = n_epi;
   h->seg_pro = n_top - n_epi;
   h->seg_cb = n_body - h->seg_ce;
-  h->seg_it = n_it0;   // kernels per Arnoldi step (the last step of a cycle has one fewer)
+  h->seg_it = n_it0;   // kernels per Arnoldi step 
   return CELL_OK;
 }
 

@@ -212,11 +212,6 @@ void resid_df(const float* xh, const float* xl, i64 xs, const double* b, i64 bs,
               int nrhs, const int* active, cudaStream_t s);
 // xh = fp32(x), xl = fp32(x - xh) for n values
 void split_f64(const double* x, float* xh, float* xl, i64 n, cudaStream_t s);
-// x64 += sc[q] * d; xh = fp32(x64), xl = fp32(x64 - xh)
-template <typename T> void axpy_split(double* x, float* xh, float* xl, i64 xs, const T* d, i64 ds,
-                                      i64 len, const double* sc, int nrhs, const int* active,
-                                      cudaStream_t s);
-
 // Tensor-core (tcgen05, 3xTF32) full-operator apply (apply_tc.cu); the grid
 // must satisfy tc_shape_ok.  err counts bounded-wait expiries.  The tables
 // (element matrix in the operand layout, hi and lo TF32 parts; gather
@@ -328,37 +323,37 @@ template <typename T> void multidot(const T* V, i64 vstride, i64 rstride, int nv
 // out[q*nvmax + i] (+)= sum over blocks of partial
 void reduce_partials(const double* partial, int nblk, int nv, int nvmax, double* out, int accumulate,
                      int nrhs, const int* active, cudaStream_t s);
-// w -= sum_i h[q*nvmax+i] V_i ; then (mode 1) partial dots <V_i,w> or (mode 2) partial |w|^2
-template <typename T> void update(const T* V, i64 vstride, i64 rstride, int nv, const double* h,
-                                  int nvmax, T* w, i64 wstride, i64 len, int mode, double* partial,
-                                  int nblk, int nrhs, const int* active, cudaStream_t s);
-// w -= sum_i h[q*nvmax+i] V_i fused with the next pass's partial dots <V_i, w>
-// (partial[..*nvmax + i], i < nv) and |w|^2 (partial[..*nvmax + nv]); nv <= 63
-template <typename T> void update_dots(const T* V, i64 vstride, i64 rstride, int nv, const double* h,
-                                       int nvmax, T* w, i64 wstride, i64 len, double* partial,
-                                       int nblk, int nrhs, const int* active, cudaStream_t s);
-template <typename T> void scale_vec(T* w, i64 wstride, i64 len, const double* sc, int nrhs,
-                                     cudaStream_t s);
-template <typename T> void lincomb(const T* V, i64 vstride, i64 rstride, const double* y,
-                                   const int* kcount, int nvmax, T* u, i64 ustride, i64 len,
-                                   int nrhs, const int* active, cudaStream_t s);
-void givens_step(double* H, double* cs, double* sn, double* g, const double* hcol,
-                 const double* hnorm2, int j, int m, int* active, double* resid, const double* tolabs,
-                 double* invscale, int* kcount, int nrhs, cudaStream_t s);
-void backsolve(const double* H, const double* g, const int* kcount, int m, double* y, int nrhs,
+// One Arnoldi step of every active load (gs.cu): w = V_{j+1} is orthogonalised
+// against V_0 .. V_j, normalised (approximately, see nu2) and the least-squares
+// problem updated.  value of vector i, load q: V[i * vstride + q * len ..].
+template <typename T>
+struct GsArgs {
+  T* V;
+  i64 vstride, len;
+  double* partial;            // 9 kNvMax nblk
+  int nblk;                   // gs_blocks(len)
+  double *gram, *nu2;         // [load][kNvMax][kNvMax] Gram rows, [load][kNvMax] squared norms
+  double *coef, *hcol;        // [load][kNvMax + 1], [load][kNvMax]
+  double *H, *cs, *sn, *g, *resid;
+  const double* tolabs;
+  int *active, *kcount, *ticket;
+  int m, nrhs;
+};
+int gs_blocks(i64 len);
+// set_next: the step runs inside a solve graph and sets the condition of the next one
+template <typename T> void gs_step(const GsArgs<T>& a, int j, cudaGraphConditionalHandle next, bool set_next,
+                                   cudaStream_t s);
+// x += sum_i y_i Z_i (FP64); FP32 also splits x into xh + xl
+template <typename T> void gs_solution(const T* Z, i64 vstride, i64 len, const double* y, const int* kcount, double* x,
+                                       float* xh, float* xl, int nrhs, const int* ran, cudaStream_t s);
+// least squares of the cycle: y for the stored (approximately normalised) directions
+void backsolve(const double* H, const double* g, const double* nu2, const int* kcount, int m, double* y, int nrhs,
                const int* mask, cudaStream_t s);
-// reorth[q] = active[q] && |w_new|^2 < |w_old|^2 / 2 (|w_old|^2 in hcol[q][j+1])
-void reorth_flag(const double* hcol, const double* hnorm2, int j, const int* active, int* reorth,
-                 int nrhs, cudaStream_t s);
-void start_cycle(const double* beta2, double* g, int m, int* active, const int* want, double* resid,
+void start_cycle(const double* beta2, double* g, double* nu2, int m, int* active, const int* want, double* resid,
                  double* invscale, const double* tolabs, int* kcount, int nrhs, cudaStream_t s);
-// v32[q] = (float)(r64[q] * sc[q])   or  x64[q] += sc[q] * d32[q]
+// v32[q] = (float)(r64[q] * sc[q])
 void to_f32_scaled(const double* r, i64 rs, float* v, i64 vs, i64 len, const double* sc, int nrhs,
                    const int* active, cudaStream_t s);
-template <typename T> void axpy_f64(double* x, i64 xs, const T* d, i64 ds, i64 len, const double* sc,
-                                    int nrhs, const int* active, cudaStream_t s);
-template <typename T> void fill(T* p, i64 n, T v, cudaStream_t s);
-
 // ---- device-side control of a whole-solve graph (solvectl.cu) ---------------------
 struct CtlParams {
   double tol;      // outer relative tolerance
@@ -376,7 +371,6 @@ void refine_ctl(const double* bn2, const double* rn2, const double* bfloor, cons
                 double* tolabs, double* relres, const int* iters, int* ctl, cudaGraphConditionalHandle cond,
                 cudaStream_t s);
 void cycle_handles(const int* active, int* ran, const IterHandles& H, cudaStream_t s);
-void next_step(const int* active, cudaGraphConditionalHandle next, cudaStream_t s);
 void accum_iters(int* iters, const int* kcount, const int* ran, int* ctl, cudaStream_t s);
 void ctl_reset(int* ctl, int* iters, cudaStream_t s);
 // v[q] = r[q] * sc[q] (FP64, nrhs vectors of len values)

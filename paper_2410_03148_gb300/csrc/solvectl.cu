@@ -65,13 +65,6 @@ __global__ void k_cycle_handles(const int* active, int* ran, const IterHandles H
   for (int j = 1; j < H.m; ++j) cudaGraphSetConditional(H.h[j], 0u);
 }
 
-__global__ void k_next_step(const int* active, cudaGraphConditionalHandle next) {
-  if (threadIdx.x != 0) return;
-  int any = 0;
-  for (int q = 0; q < 9; ++q) any |= active[q];
-  cudaGraphSetConditional(next, any ? 1u : 0u);
-}
-
 // End of a cycle: iteration counts of the loads that ran, and the number of
 // Arnoldi steps the graph executed (the largest count).
 __global__ void k_accum_iters(int* iters, const int* kcount, const int* ran, int* ctl) {
@@ -110,10 +103,6 @@ void refine_ctl(const double* bn2, const double* rn2, const double* bfloor, cons
 
 void cycle_handles(const int* active, int* ran, const IterHandles& H, cudaStream_t s) {
   note_launch(), k_cycle_handles<<<1, 32, 0, s>>>(active, ran, H);
-}
-
-void next_step(const int* active, cudaGraphConditionalHandle next, cudaStream_t s) {
-  note_launch(), k_next_step<<<1, 32, 0, s>>>(active, next);
 }
 
 void accum_iters(int* iters, const int* kcount, const int* ran, int* ctl, cudaStream_t s) {

@@ -118,3 +118,24 @@ def test_rediscretised_hierarchy_options(shape, opt):
     assert max(st["rel_residual"]) <= 1e-10
     for got, key in zip(cell.homogenise(), ("C", "e", "kappa")):
         assert np.abs(got - ref[key]).max() < 1e-8 * np.abs(ref[key]).max(), key
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("opt", [{"restart": 3}, {"restart": 17, "inner_tol": 1e-7}, {"restart": 40, "inner_tol": 1e-12, "max_refine": 4},
+                                 {"restart": 63, "inner_tol": 1e-12, "max_refine": 3, "cheb_degree": 1, "vcycles_phi": 1}])
+def test_arnoldi_step_lengths(precision, opt):
+    """Every form of the Gram-Schmidt kernels: up to 4, 8 and 16 basis vectors in
+    registers, more read twice (an inner tolerance below FP32 rounding keeps a
+    cycle going to its restart length), short restarts, one and two entries
+    per lane of the forward substitution (up to 63 vectors)."""
+    from paper_2410_03148_gb300 import Cell
+    from oracle import ersatz
+    shape = (7, 10, 9)
+    M = cellgen.pzt5h_class()
+    phi = cellgen.gaussian_levelset(shape, seed=6)
+    ref = fem.solve_cell(ersatz.rho_from_levelset(phi), *M)
+    cell = Cell(torch.as_tensor(phi, device="cuda:0"), M, kind="phi", **{"precision": precision, "max_iter": 2000, **opt})
+    st = cell.solve()
+    assert max(st["rel_residual"]) <= 1e-10
+    for got, key in zip(cell.homogenise(), ("C", "e", "kappa")):
+        assert np.abs(got - ref[key]).max() < 1e-8 * np.abs(ref[key]).max(), key
