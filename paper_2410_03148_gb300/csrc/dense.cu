@@ -4,8 +4,9 @@
 // over the whole chip.  On the host the FP64 factorisation of the default
 // coarsest level (192 unknowns) took 5 ms per design, half of an 8^3 design
 // step.  FP64 elimination in one block would take 1.7 ms (n^3 multiply-adds at
-// two per clock); the FP32 one takes 0.05 ms and Newton-Schulz squares its
-// residual.
+// two per clock); the FP32 one takes 0.17 ms (0.9 us a pivot, bound by its
+// chain of barrier, shared-memory reads and update) and Newton-Schulz squares
+// its residual.
 #include "kernels.cuh"
 
 namespace cell {
@@ -45,23 +46,28 @@ __global__ void k_dense_rows(const T* __restrict__ rho, const double* __restrict
 // Null-space regularisation (mean of every component, scaled by the mean
 // diagonal) and X = A^-1 in FP32: in-place Gauss-Jordan without pivoting (A is
 // symmetric positive definite), a 32 x 32 block of threads with entry
-// (ty + 32 a, tx + 32 b) in register (a, b).
+// (ty + 32 a, tx + 32 b) in register (a, b), TILE = ceil(n / 32).  The pivot row
+// and column of the next step are written to the other buffer right after the
+// update, so a step has one barrier.
+template <int TILE>
 __global__ void __launch_bounds__(1024, 1)
-k_dense_invert(double* __restrict__ A, double* __restrict__ X, int n, int nn, int nc) {
-  __shared__ float row[kMaxN], col[kMaxN];
+k_dense_invert(double* __restrict__ A, double* __restrict__ X, int n, int nn) {
+  __shared__ float row[2][32 * TILE], col[2][32 * TILE];
   __shared__ double mean;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
+  if (ty == 0) {
     double tr = 0.0;
-    for (int i = 0; i < n; ++i) tr += A[(size_t)i * n + i];
-    mean = tr / n / nn;
+    for (int i = tx; i < n; i += 32) tr += A[(size_t)i * n + i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+    if (tx == 0) mean = tr / n / nn;
   }
   __syncthreads();
-  float a[kTile][kTile];
+  float a[TILE][TILE];
 #pragma unroll
-  for (int p = 0; p < kTile; ++p)
+  for (int p = 0; p < TILE; ++p)
 #pragma unroll
-    for (int q = 0; q < kTile; ++q) {
+    for (int q = 0; q < TILE; ++q) {
       const int i = ty + 32 * p, j = tx + 32 * q;
       a[p][q] = 0.f;
       if (i < n && j < n) {
@@ -73,45 +79,66 @@ k_dense_invert(double* __restrict__ A, double* __restrict__ X, int n, int nn, in
         a[p][q] = (float)v;
       }
     }
-  for (int k = 0; k < n; ++k) {
+  // Pivot row and column into shared memory; their registers are cleared and
+  // the pivot's entries set to 1 (row) and -1 (column), so that the rank-1
+  // update a - f r gives every case: the pivot row becomes r, the pivot column
+  // -f piv, the pivot piv.
+  __shared__ float pivot[2];
+  auto publish = [&](int k) {
     const int kt = k & 31, kb = k >> 5;
+    float* rk = row[k & 1];
+    float* ck = col[k & 1];
+    if (ty == kt) {
 #pragma unroll
-    for (int p = 0; p < kTile; ++p) {
-      if (p != kb) continue;
-      if (ty == kt) {
+      for (int p = 0; p < TILE; ++p)
+        if (p == kb) {
 #pragma unroll
-        for (int q = 0; q < kTile; ++q) row[tx + 32 * q] = a[p][q];
-      }
+          for (int q = 0; q < TILE; ++q) {
+            if (q == kb && tx == kt) {
+              pivot[k & 1] = a[p][q];
+              rk[tx + 32 * q] = 1.f;
+            } else {
+              rk[tx + 32 * q] = a[p][q];
+            }
+            a[p][q] = 0.f;
+          }
+        }
     }
     if (tx == kt) {
 #pragma unroll
-      for (int p = 0; p < kTile; ++p)
+      for (int q = 0; q < TILE; ++q)
+        if (q == kb) {
 #pragma unroll
-        for (int q = 0; q < kTile; ++q)
-          if (q == kb) col[ty + 32 * p] = a[p][q];
+          for (int p = 0; p < TILE; ++p) {
+            // the pivot row's owner has cleared its register already
+            ck[ty + 32 * p] = p == kb && ty == kt ? -1.f : a[p][q];
+            a[p][q] = 0.f;
+          }
+        }
     }
-    __syncthreads();
-    const float piv = 1.f / row[k];
-    float r[kTile];
+  };
+  publish(0);
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
+    const float* rk = row[k & 1];
+    const float* ck = col[k & 1];
+    const float piv = 1.f / pivot[k & 1];
+    float r[TILE];
 #pragma unroll
-    for (int q = 0; q < kTile; ++q) r[q] = row[tx + 32 * q] * piv;
+    for (int q = 0; q < TILE; ++q) r[q] = rk[tx + 32 * q] * piv;
 #pragma unroll
-    for (int p = 0; p < kTile; ++p) {
-      const float f = col[ty + 32 * p];
-      const bool own = p == kb && ty == kt;
+    for (int p = 0; p < TILE; ++p) {
+      const float f = -ck[ty + 32 * p];
 #pragma unroll
-      for (int q = 0; q < kTile; ++q) {
-        const bool pc = q == kb && tx == kt;
-        // pivot row: scaled; pivot column: -f piv; pivot: piv; else rank-1 update
-        a[p][q] = own ? (pc ? piv : r[q]) : (pc ? -f * piv : fmaf(-f, r[q], a[p][q]));
-      }
+      for (int q = 0; q < TILE; ++q) a[p][q] = fmaf(f, r[q], a[p][q]);
     }
+    if (k + 1 < n) publish(k + 1);
     __syncthreads();
   }
 #pragma unroll
-  for (int p = 0; p < kTile; ++p)
+  for (int p = 0; p < TILE; ++p)
 #pragma unroll
-    for (int q = 0; q < kTile; ++q) {
+    for (int q = 0; q < TILE; ++q) {
       const int i = ty + 32 * p, j = tx + 32 * q;
       if (i < n && j < n) X[(size_t)i * n + j] = (double)a[p][q];
     }
@@ -167,7 +194,16 @@ void dense_invert(const T* rho, const double* K, int nc, int nx, int ny, int nz,
   double *A = work, *X = work + n2, *R = work + 2 * n2, *Y = work + 3 * n2;
   cudaMemsetAsync(dev, 0, sizeof(unsigned), s);
   note_launch(), k_dense_rows<T><<<n, n < 256 ? (n + 31) / 32 * 32 : 256, 0, s>>>(rho, K, nc, nx, ny, nz, A);
-  note_launch(), k_dense_invert<<<1, 1024, 0, s>>>(A, X, n, nn, nc);
+  note_launch();
+  switch ((n + 31) / 32) {
+    case 1: k_dense_invert<1><<<1, 1024, 0, s>>>(A, X, n, nn); break;
+    case 2: k_dense_invert<2><<<1, 1024, 0, s>>>(A, X, n, nn); break;
+    case 3: k_dense_invert<3><<<1, 1024, 0, s>>>(A, X, n, nn); break;
+    case 4: k_dense_invert<4><<<1, 1024, 0, s>>>(A, X, n, nn); break;
+    case 5: k_dense_invert<5><<<1, 1024, 0, s>>>(A, X, n, nn); break;
+    case 6: k_dense_invert<6><<<1, 1024, 0, s>>>(A, X, n, nn); break;
+    default: k_dense_invert<kTile><<<1, 1024, 0, s>>>(A, X, n, nn); break;
+  }
   const dim3 g((unsigned)((n + 15) / 16), (unsigned)((n + 15) / 16));
   note_launch(), k_dense_mul<T><<<g, 256, 0, s>>>(A, X, R, n, 0, nullptr, nullptr);
   note_launch(), k_dense_mul<T><<<g, 256, 0, s>>>(X, R, Y, n, 1, nullptr, nullptr);
