@@ -260,6 +260,7 @@ struct cell_handle {
   double h[3];
   double K0[1024], S0[64], Z[288], F[288], H0e[81];
   bool modal = false;            // mm2 material: operators in modal form
+  double Km[1024];               // modal matrix of K0
   ModalSet<float> m32;
   ModalSet<double> m64;
   unsigned* dense_dev = nullptr;      // residuals of the two coarsest inverses (float bits)
@@ -1296,12 +1297,12 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
   }
   h->modal = cellhost::is_mm2(d->C, d->e, d->kappa);
   if (h->modal) {
-    double Km[1024], Sm[64];
-    cellhost::modal_matrix(h->K0, 4, Km);
+    double Sm[64];
+    cellhost::modal_matrix(h->K0, 4, h->Km);
     cellhost::modal_matrix(h->S0, 1, Sm);
-    fill_modal_set(Km, Sm, h->m32);
-    fill_modal_set(Km, Sm, h->m64);
-    fill_modal<4, 4, cell::DF>(Km, 4, 0, h->mdf, [](double v) {
+    fill_modal_set(h->Km, Sm, h->m32);
+    fill_modal_set(h->Km, Sm, h->m64);
+    fill_modal<4, 4, cell::DF>(h->Km, 4, 0, h->mdf, [](double v) {
       const float hi = (float)v;
       return cell::DF{hi, (float)(v - (double)hi)};
     });
@@ -1831,6 +1832,31 @@ void run_sensitivity(cell_handle* h, const cell::SensParams& P, T* g) {
   cell::SensModes<T> M;
   sens_modes<T>(h, P, &Q, &M);
   void* work = h->d.opt.precision == CELL_MIXED_FP32 ? (void*)h->kf.V : (void*)h->kd.V;
+  if (h->modal) {
+    cell::SensModal<T> S;
+    std::memset(&S, 0, sizeof(S));
+    const double* Km = h->Km;
+    const cell::SensPairTable pairs = cell::sens_pair_table();
+    for (int n = 0; n < cell::kSensPairs; ++n) {
+      const int a = pairs.p[n].a, b = pairs.p[n].b;
+      const double v = Km[((a & 7) * 4 + (a >> 3)) * 32 + (b & 7) * 4 + (b >> 3)];
+      S.k[n] = (T)(a == b ? v : 2.0 * v);
+    }
+    // the loads are affine: their modes are the sums over the 4 edges along an axis
+    for (int d = 0; d < 3; ++d)
+      for (int c = 0; c < 4; ++c)
+        for (int m = 0; m < Q.R; ++m) {
+          double z = 0.0;
+          for (int a = 0; a < 8; ++a)
+            for (int I = 0; I < 9; ++I)
+              z += ((a >> d) & 1 ? 1.0 : -1.0) * P.Z[(4 * a + c) * 9 + I] * Q.q[I * 9 + m];
+          S.zq[(d * 4 + c) * 9 + m] = (T)z;
+        }
+    std::memcpy(S.lam, M.lam, sizeof(S.lam));
+    S.R = Q.R;
+    cell::sensitivity_modal<T>(h->x64, Q, S, static_cast<T*>(work), g, h->nx, h->ny, h->nz, h->st);
+    return;
+  }
   cell::sensitivity<T>(h->x64, h->rho64, Q, M, static_cast<T*>(work), g, h->nx, h->ny, h->nz, 0, h->st);
 }
 }  // namespace

@@ -18,6 +18,14 @@ void report_error(const char* what, cudaError_t e);
 extern std::atomic<long long> g_launches;
 inline void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
+// Mirror parity of dof (component c, mode m): a displacement component and
+// its own axis' difference flip together, the potential with z.  An mm2
+// material couples only dofs of equal parity.
+__host__ __device__ constexpr int modal_parity(int c, int m) { return m ^ (c == 0 ? 1 : (c == 1 ? 2 : 4)); }
+__host__ __device__ constexpr bool modal_couples(int c, int m, int c2, int m2) {
+  return modal_parity(c, m) == modal_parity(c2, m2);
+}
+
 // Leading dimension of the per-load Krylov scalars (Gram-Schmidt columns,
 // partial sums); bounds the GMRES restart length.
 constexpr int kNvMax = 64;
@@ -44,6 +52,40 @@ template <typename T>
 struct SensModes {
   T ku[1024];     // upper triangle of K0 (row-major), off-diagonal entries doubled
   T zq[32 * 9];   // affine part of the modes at local dof a: (Zbar Q)[a*9 + m]
+  T lam[9];
+  int R;
+};
+
+// The same in element modes (mm2 materials, modal.cuh): k = upper triangle of
+// K0's modal matrix by class, off-diagonal entries doubled, in the order of
+// sens_pairs; the affine part has constant strains only: zq[(i 4 + c) 9 + m]
+// of the mode "difference along i".
+struct SensPairIndex {
+  unsigned char a, b;   // dofs 8 c + mode, a <= b
+};
+constexpr int kSensPairs = 55;
+// Coupled pairs (a <= b) of the 28 modal dofs in row order; compile-time.
+struct SensPairTable {
+  SensPairIndex p[kSensPairs];
+};
+__host__ __device__ constexpr int modal_bits(int m) { return (m & 1) + ((m >> 1) & 1) + (m >> 2); }
+constexpr SensPairTable sens_pair_table() {
+  SensPairTable t{};
+  int n = 0;
+  for (int a = 0; a < 32; ++a)
+    for (int b = a; b < 32; ++b) {
+      const int ma = a & 7, mb = b & 7;
+      if (ma == 0 || mb == 0 || modal_bits(ma) != modal_bits(mb) || !modal_couples(a >> 3, ma, b >> 3, mb)) continue;
+      t.p[n].a = (unsigned char)a;
+      t.p[n].b = (unsigned char)b;
+      ++n;
+    }
+  return t;
+}
+template <typename T>
+struct SensModal {
+  T k[kSensPairs];
+  T zq[12 * 9];
   T lam[9];
   int R;
 };
@@ -100,13 +142,6 @@ struct ApplyArgs {
 struct DF {         // unevaluated pair h + l
   float h, l;
 };
-// Mirror parity of dof (component c, mode m): a displacement component and
-// its own axis' difference flip together, the potential with z.  An mm2
-// material couples only dofs of equal parity.
-__host__ __device__ constexpr int modal_parity(int c, int m) { return m ^ (c == 0 ? 1 : (c == 1 ? 2 : 4)); }
-__host__ __device__ constexpr bool modal_couples(int c, int m, int c2, int m2) {
-  return modal_parity(c, m) == modal_parity(c2, m2);
-}
 enum ModalKind { MK_FULL = 0, MK_UU = 1, MK_PU = 2, MK_SS = 3 };   // Ahat, A, B, Sbar
 enum ModalMode {
   MM_APPLY = 0,   // y = A x
@@ -419,6 +454,9 @@ void gram9(const double* u, const double* v, i64 nn, double* partial, int nblk, 
 // out[0] = sum of x[0..n) (or of the squares)  (device scalar)
 void sum_reduce(const double* x, i64 n, double* partial, int nblk, double* out, cudaStream_t s,
                 int squares = 0);
+// Element sensitivities of mm2 materials; as sensitivity (no rho factor).
+template <typename T> void sensitivity_modal(const double* y, const SensQ& Q, const SensModal<T>& P, T* xwork, T* g,
+                                             int nx, int ny, int nz, cudaStream_t s);
 // g_e = (rho_e if times_rho) * sum_IJ G_IJ W_e^I . K0 W_e^J, W = Zbar + y_e,
 // evaluated as sum_m lam_m X^m.K0 X^m; xwork holds Q.R x 8 x nn floats (T =
 // float: FP32 pairs of the mode fields) or Q.R x 4 x nn doubles.
