@@ -76,11 +76,20 @@ template <>
 struct Pair<float> {
   float2 p;
 };
+template <>
+struct Pair<DF> {
+  float2 h, l;
+};
 template <typename V> __device__ __forceinline__ V sum_of(const Pair<V>& a) { return a.s; }
 template <typename V> __device__ __forceinline__ V dif_of(const Pair<V>& a) { return a.d; }
 __device__ __forceinline__ float sum_of(const Pair<float>& a) { return a.p.x; }
 __device__ __forceinline__ float dif_of(const Pair<float>& a) { return a.p.y; }
+__device__ __forceinline__ DF sum_of(const Pair<DF>& a) { return {a.h.x, a.l.x}; }
+__device__ __forceinline__ DF dif_of(const Pair<DF>& a) { return {a.h.y, a.l.y}; }
 template <typename V> __device__ __forceinline__ Pair<V> mk(V s, V d) { return {s, d}; }
+template <> __device__ __forceinline__ Pair<DF> mk<DF>(DF s, DF d) {
+  return {make_float2(s.h, d.h), make_float2(s.l, d.l)};
+}
 template <> __device__ __forceinline__ Pair<float> mk<float>(float s, float d) { return {make_float2(s, d)}; }
 template <typename V> __device__ __forceinline__ Pair<V> padd(const Pair<V>& a, const Pair<V>& b) {
   return {vadd(a.s, b.s), vadd(a.d, b.d)};
@@ -99,6 +108,27 @@ __device__ __forceinline__ Pair<float> psub(const Pair<float>& a, const Pair<flo
 }
 __device__ __forceinline__ Pair<float> pmul(float k, const Pair<float>& a) {
   return {__fmul2_rn(make_float2(k, k), a.p)};
+}
+
+// The error-free sums of vadd and vsub, two at a time.
+__device__ __forceinline__ float2 minus(const float2 b, const float2 a) {   // a - b
+  return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+}
+__device__ __forceinline__ Pair<DF> padd(const Pair<DF>& a, const Pair<DF>& b) {
+  const float2 s = __fadd2_rn(a.h, b.h), t = minus(a.h, s);
+  const float2 e = __fadd2_rn(minus(minus(t, s), a.h), minus(t, b.h));
+  return {s, __fadd2_rn(__fadd2_rn(a.l, b.l), e)};
+}
+__device__ __forceinline__ Pair<DF> psub(const Pair<DF>& a, const Pair<DF>& b) {
+  const float2 s = minus(b.h, a.h), t = minus(a.h, s);
+  const float2 e = minus(__fadd2_rn(b.h, t), minus(minus(t, s), a.h));
+  return {s, __fadd2_rn(minus(b.l, a.l), e)};
+}
+__device__ __forceinline__ Pair<DF> pmul(DF k, const Pair<DF>& a) {
+  const float2 kh = make_float2(k.h, k.h), kl = make_float2(k.l, k.l);
+  const float2 p = __fmul2_rn(kh, a.h);
+  const float2 e = __ffma2_rn(kh, a.h, make_float2(-p.x, -p.y));
+  return {p, __ffma2_rn(kh, a.l, __ffma2_rn(kl, a.h, e))};
 }
 
 // ---- element contraction ------------------------------------------------------

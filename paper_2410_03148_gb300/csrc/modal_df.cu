@@ -32,7 +32,11 @@ struct DfIO {
   }
 };
 
-constexpr int kRows = 2, kBlocksPerSM = 2;
+// Rows per strip at 128^3 / 64^3 / 32^3 with nine loads (us): one 3717 / 546 / 82,
+// two 3845 / 524 / 84 (4176 / 557 / 88 before the sums of the x pairs became
+// packed instructions; the corner form took 8300 at 128^3).  Both spill at 255
+// registers (184 and 560 bytes); the arithmetic alone would take about 1.5 ms.
+constexpr int kRows = 1, kBlocksPerSM = 2;
 
 __global__ void __launch_bounds__(modal::kThreads, kBlocksPerSM)
 k_modal_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs, const double* __restrict__ b, i64 bs,
