@@ -2273,7 +2273,7 @@ int cell_hilbert_velocity(cell_handle* h, double alpha, const double* dJ, const 
   for (int i = 0; i < ncons; ++i)
     if (!dC[i] || !std::isfinite(C[i])) return CELL_EINVAL;
   if (!std::isfinite(wJ) || !std::isfinite(wC)) return CELL_EINVAL;
-  // workspace: 4 (1 + ncons) nn doubles of the Krylov basis ((m + 1) x 9 x 4 nn values)
+  // workspace: 2 (1 + ncons) nn doubles of the Krylov basis ((m + 1) x 9 x 4 nn values)
   const bool mixed = h->d.opt.precision == CELL_MIXED_FP32;
   if ((mixed ? (h->d.opt.restart + 1) / 2 : h->d.opt.restart + 1) < 1) return CELL_EINVAL;
   double* work = mixed ? reinterpret_cast<double*>(h->kf.V) : h->kd.V;

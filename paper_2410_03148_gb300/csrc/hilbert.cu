@@ -35,46 +35,135 @@ namespace {
 constexpr int kB = 256;
 constexpr int kMaxVec = 1 + kHilbertMaxCons;
 
+// The stencil is symmetric along every axis: c[x + 2 y + 4 z] is the
+// coefficient of the neighbours at distance 1 along the axes whose bit is set.
 struct Stencil {
-  double c[27];   // coefficient of neighbour (dx, dy, dz) at (dx + 1) + 3 (dy + 1) + 9 (dz + 1)
+  double c[8];
 };
 
-// x = 0 (implicit), r = d, p = d / theta for every vector (grid y = vector)
-__global__ void k_cheb_init(const double* const* __restrict__ rhs, double* __restrict__ r,
-                            double* __restrict__ p, double* __restrict__ x, i64 nn, double inv_theta) {
+// x_1 = d / theta for every vector (grid y = vector)
+__global__ void k_cheb_init(const double* const* __restrict__ rhs, double* __restrict__ x, i64 nn, double inv_theta) {
   const int v = blockIdx.y;
   const double* d = rhs[v];
-  for (i64 n = (i64)blockIdx.x * blockDim.x + threadIdx.x; n < nn; n += (i64)gridDim.x * blockDim.x) {
-    const double b = d[n];
-    r[v * nn + n] = b;
-    p[v * nn + n] = b * inv_theta;
-    x[v * nn + n] = 0.0;
+  for (i64 n = (i64)blockIdx.x * blockDim.x + threadIdx.x; n < nn; n += (i64)gridDim.x * blockDim.x)
+    x[v * nn + n] = d[n] * inv_theta;
+}
+
+// One Chebyshev step in three-term form,
+//   x_{k+1} = x_k + ca (x_k - x_{k-1}) + cb (d - A x_k)
+//           = S x_k - ca x_{k-1} + cb d,   S = (1 + ca) I - cb A,
+// x_{k+1} over x_{k-1} (first: x_0 = 0, written only).  FP64 arithmetic (1/64
+// rate) bounds it.
+//
+// Large grids: a warp marches a strip of kRows rows by 30 columns (lanes 1 ..
+// 30; lanes 0 and 31 are halo) through z and adds the two neighbours along x,
+// the rows of a strip along y and the planes along z once: 15 operations per
+// node.  The columns of all strips form one sequence of nx + 2 positions each,
+// cut into windows of 30.
+constexpr int kRows = 4, kOut = 30, kStepThreads = 128, kStepWarps = kStepThreads / 32;
+
+__global__ void __launch_bounds__(kStepThreads)
+k_cheb_step(const __grid_constant__ Stencil S, const double* const* __restrict__ rhs, const double* __restrict__ xin,
+            double* xio, int first, int nx, int ny, int nz, int L, double ca, double cb) {
+  const int lane = threadIdx.x & 31;
+  const int rl = nx + 2, strips = (ny + kRows - 1) / kRows;
+  const int p0 = (int)(blockIdx.x * kStepWarps + (threadIdx.x >> 5)) * kOut;
+  if (p0 >= strips * rl - 2) return;   // warp-uniform
+  const int p = min(p0 + lane, strips * rl - 1);
+  const int strip = p / rl, xi = p - strip * rl - 1;
+  const bool vx = lane >= 1 && lane <= kOut && p0 + lane == p && xi >= 0 && xi < nx;
+  const int i = xi < 0 ? nx - 1 : (xi >= nx ? 0 : xi);
+  const int j0 = strip * kRows;
+  unsigned ro[kRows + 2];
+#pragma unroll
+  for (int r = 0; r < kRows + 2; ++r) {
+    int j = j0 - 1 + r;   // at most ny + kRows - 1: two subtractions wrap it
+    j = j < 0 ? j + ny : j;
+    j = j >= ny ? j - ny : j;
+    j = j >= ny ? j - ny : j;
+    ro[r] = (unsigned)(j * nx + i);
+  }
+  const unsigned nxy = (unsigned)(nx * ny);
+  const i64 nn = (i64)nxy * nz;
+  const double* X = xin + blockIdx.y * nn;
+  double* Y = xio + blockIdx.y * nn;
+  const double* D = rhs[blockIdx.y];
+  const int z0 = blockIdx.z * L, Lc = min(L, nz - z0);
+  // planes z0 - 1 .. z0 + Lc; U: in-plane part of the plane before plus the z
+  // part of the one before that; W: z part of the plane before
+  double U[kRows], W[kRows], vn[kRows + 2];
+  unsigned zo = (unsigned)(z0 == 0 ? nz - 1 : z0 - 1) * nxy, zb = 0;
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) U[r] = W[r] = 0.0;
+#pragma unroll
+  for (int r = 0; r < kRows + 2; ++r) vn[r] = __ldg(X + zo + ro[r]);
+#pragma unroll 1
+  for (int t = -1; t <= Lc; ++t) {
+    const unsigned zn = zo + nxy == nxy * (unsigned)nz ? 0 : zo + nxy;
+    double v[kRows + 2], xs[kRows + 2], d[kRows], xp[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows + 2; ++r) {
+      v[r] = vn[r];
+      vn[r] = __ldg(X + zn + ro[r]);   // the plane after the last is read and not used
+    }
+    if (t > 0 && vx) {
+#pragma unroll
+      for (int r = 0; r < kRows; ++r) {
+        if (j0 + r >= ny) continue;
+        d[r] = __ldg(D + zb + ro[r + 1]);
+        xp[r] = first ? 0.0 : Y[zb + ro[r + 1]];
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows + 2; ++r)
+      xs[r] = __shfl_up_sync(0xffffffffu, v[r], 1) + __shfl_down_sync(0xffffffffu, v[r], 1);
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const double P = v[r + 1], Xs = xs[r + 1], Ys = v[r] + v[r + 2], XY = xs[r] + xs[r + 2];
+      const double w = fma(S.c[7], XY, fma(S.c[6], Ys, fma(S.c[5], Xs, S.c[4] * P)));
+      const double ax = U[r] + w;   // S x on the plane before
+      if (t > 0 && vx && j0 + r < ny)
+        Y[zb + ro[r + 1]] = fma(-ca, xp[r], fma(cb, d[r], ax));
+      U[r] = fma(S.c[3], XY, fma(S.c[2], Ys, fma(S.c[1], Xs, fma(S.c[0], P, W[r]))));
+      W[r] = w;
+    }
+    zb = zo;
+    zo = zn;
   }
 }
 
-// One Chebyshev step per node: x += p, r -= A p, p_new = a p + b r_new
-// (p read from pin, written to pout: neighbours read the old direction).
-__global__ void __launch_bounds__(kB)
-k_cheb_step(const __grid_constant__ Stencil S, const double* __restrict__ pin, double* __restrict__ pout,
-            double* __restrict__ r, double* __restrict__ x, int nx, int ny, int nz, double ca, double cb) {
-  const i64 nxy = (i64)nx * ny, nn = nxy * nz;
-  const i64 n = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+// Small grids: one thread per node, 27 products in the grouped order of the
+// symmetric stencil (19 additions and 8 products).
+__global__ void __launch_bounds__(kStepThreads)
+k_cheb_step_node(const __grid_constant__ Stencil S, const double* const* __restrict__ rhs, const double* __restrict__ xin,
+                 double* xio, int first, int nx, int ny, int nz, double ca, double cb) {
+  const int n = blockIdx.x * kStepThreads + threadIdx.x, nxy = nx * ny, nn = nxy * nz;
   if (n >= nn) return;
-  const int v = blockIdx.y;
-  const int i = (int)(n % nx), j = (int)((n / nx) % ny), k = (int)(n / nxy);
+  const int k = n / nxy, ij = n - k * nxy, j = ij / nx, i = ij - j * nx;
   const int xo[3] = {i == 0 ? nx - 1 : i - 1, i, i == nx - 1 ? 0 : i + 1};
-  const i64 yo[3] = {(i64)(j == 0 ? ny - 1 : j - 1) * nx, (i64)j * nx, (i64)(j == ny - 1 ? 0 : j + 1) * nx};
-  const i64 zo[3] = {(i64)(k == 0 ? nz - 1 : k - 1) * nxy, (i64)k * nxy, (i64)(k == nz - 1 ? 0 : k + 1) * nxy};
-  const double* P = pin + v * nn;
-  double ap = 0.0;
+  const int yo[3] = {(j == 0 ? ny - 1 : j - 1) * nx, j * nx, (j == ny - 1 ? 0 : j + 1) * nx};
+  const int zo[3] = {(k == 0 ? nz - 1 : k - 1) * nxy, k * nxy, (k == nz - 1 ? 0 : k + 1) * nxy};
+  const i64 base = (i64)blockIdx.y * nn;
+  const double* X = xin + base;
+  const double dn = __ldg(rhs[blockIdx.y] + n);
+  const double xp = first ? 0.0 : xio[base + n];
+  // P, Xs, Ys, XY of the planes k and k - 1 + k + 1
+  double s[2][4];
 #pragma unroll
-  for (int q = 0; q < 27; ++q) ap = fma(S.c[q], P[xo[q % 3] + yo[(q / 3) % 3] + zo[q / 9]], ap);
-  const i64 o = v * nn + n;
-  const double pn = P[n];
-  x[o] += pn;
-  const double rn = r[o] - ap;
-  r[o] = rn;
-  pout[o] = ca * pn + cb * rn;
+  for (int z = 0; z < 3; ++z) {
+    double v[3][3];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) v[q / 3][q % 3] = __ldg(X + xo[q % 3] + yo[q / 3] + zo[z]);
+    const double x0 = v[0][0] + v[0][2], x1 = v[1][0] + v[1][2], x2 = v[2][0] + v[2][2];
+    const double t[4] = {v[1][1], x1, v[0][1] + v[2][1], x0 + x2};
+    const int o = z == 1 ? 0 : 1;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s[o][c] = z == 2 ? s[o][c] + t[c] : t[c];
+  }
+  double ax = 0.0;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) ax = fma(S.c[c], s[c >> 2][c & 3], ax);
+  xio[base + n] = fma(-ca, xp, fma(cb, dn, ax));
 }
 
 // partial[(a * nblk + blk) * kNvMax + b] = block sum of g_a . d_b
@@ -166,42 +255,56 @@ int hilbert_velocity(int nx, int ny, int nz, double alpha, const double* dJ, con
   int iters = q <= 0.0 ? 1 : (int)std::ceil(std::log(1e-13 / 2.0) / std::log(q));
   iters = std::max(1, std::min(iters, 20000));
   const bool flat = !(delta > 1e-14 * theta);   // one eigenvalue: x = d / theta in one step
-  // stencil of A
+  // stencil of A: coefficient of a neighbour at distance (0 or 1) along the axes
   Stencil S;
   double sx[3], mx[3], sy[3], my[3], sz[3], mz[3];
   stencils_1d(h[0], sx, mx);
   stencils_1d(h[1], sy, my);
   stencils_1d(h[2], sz, mz);
-  for (int dz = 0; dz < 3; ++dz)
-    for (int dy = 0; dy < 3; ++dy)
-      for (int dx = 0; dx < 3; ++dx)
-        S.c[dx + 3 * dy + 9 * dz] = alpha * alpha * (sx[dx] * my[dy] * mz[dz] + mx[dx] * sy[dy] * mz[dz] +
-                                                     mx[dx] * my[dy] * sz[dz]) +
-                                    mx[dx] * my[dy] * mz[dz];
-  // workspace: x (the representers), r, p, p2: nvec x nn doubles each
+  for (int o = 0; o < 8; ++o) {
+    const int dx = (o & 1) ? 2 : 1, dy = (o & 2) ? 2 : 1, dz = (o & 4) ? 2 : 1;
+    S.c[o] = alpha * alpha * (sx[dx] * my[dy] * mz[dz] + mx[dx] * sy[dy] * mz[dz] + mx[dx] * my[dy] * sz[dz]) +
+             mx[dx] * my[dy] * mz[dz];
+  }
+  // workspace: two iterates of nvec x nn doubles
   double* x = work;
-  double* r = x + nvec * nn;
-  double* p = r + nvec * nn;
-  double* p2 = p + nvec * nn;
+  double* x2 = x + nvec * nn;
   const double* hp[kMaxVec];
   hp[0] = dJ;
   for (int i = 0; i < ncons; ++i) hp[1 + i] = dC[i];
   cudaError_t e = cudaMemcpyAsync(dptrs_dev, hp, nvec * sizeof(double*), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return CELL_ECUDA;
   const unsigned nb = (unsigned)std::min<i64>((nn + kB - 1) / kB, 4096);
-  note_launch(), k_cheb_init<<<dim3(nb, nvec), kB, 0, s>>>(dptrs_dev, r, p, x, nn, 1.0 / theta);
-  const unsigned nbs = (unsigned)((nn + kB - 1) / kB);
+  note_launch(), k_cheb_init<<<dim3(nb, nvec), kB, 0, s>>>(dptrs_dev, x, nn, 1.0 / theta);
+  // The march pays its longer serial chain back from about 4e5 node values on
+  // (us a step, node kernel against march: 96^3 x 4 200 / 151, 64^3 x 3 48 / 40,
+  // 48^3 x 3 24 / 26, 64^3 x 1 20 / 22, 30 x 33 x 27 x 2 7 / 17; before, with 27
+  // products and the direction form: 216, 53, 9);
+  // two blocks per SM, a chunk reads two planes more than it writes.
+  const bool march = nn * nvec >= 400000;
+  const i64 windows = ((i64)((ny + kRows - 1) / kRows) * (nx + 2) - 2 + kOut - 1) / kOut;
+  const i64 blocks = (windows + kStepWarps - 1) / kStepWarps;
+  i64 chunks = std::max<i64>(1, modal::sm_count() * 2 / (blocks * nvec));
+  chunks = std::min<i64>(chunks, std::min(nz, 4096));
+  const int L = (int)((nz + chunks - 1) / chunks);
+  const dim3 grid((unsigned)blocks, (unsigned)nvec, (unsigned)((nz + L - 1) / L));
+  const dim3 nodes((unsigned)((nn + kStepThreads - 1) / kStepThreads), (unsigned)nvec);
   const double s1 = flat ? 1.0 : theta / delta;
   double rho0 = 1.0 / s1;
-  for (int k = 0; k < (flat ? 1 : iters); ++k) {
-    const double rho1 = flat ? 0.0 : 1.0 / (2.0 * s1 - rho0);
-    const double ca = rho1 * rho0, cb = flat ? 0.0 : 2.0 * rho1 / delta;
-    note_launch(), k_cheb_step<<<dim3(nbs, nvec), kB, 0, s>>>(S, p, p2, r, x, nx, ny, nz, ca, cb);
-    std::swap(p, p2);
+  // x_1 = d / theta is the first of the iterations
+  for (int k = 0; k + 1 < (flat ? 1 : iters); ++k) {
+    const double rho1 = 1.0 / (2.0 * s1 - rho0);
+    const double ca = rho1 * rho0, cb = 2.0 * rho1 / delta;
+    Stencil Sk;
+    for (int o = 0; o < 8; ++o) Sk.c[o] = (o == 0 ? 1.0 + ca : 0.0) - cb * S.c[o];
+    if (march)
+      note_launch(), k_cheb_step<<<grid, kStepThreads, 0, s>>>(Sk, dptrs_dev, x, x2, k == 0, nx, ny, nz, L, ca, cb);
+    else
+      note_launch(), k_cheb_step_node<<<nodes, kStepThreads, 0, s>>>(Sk, dptrs_dev, x, x2, k == 0, nx, ny, nz, ca, cb);
+    std::swap(x, x2);
     rho0 = rho1;
   }
   if (flat) iters = 1;
-  // the last direction is not added (x_k = x_{k-1} + p_{k-1} is already the iterate)
   note_launch(), k_gram<<<dim3(nblk, nvec), kB, 0, s>>>(x, dptrs_dev, nvec, nn, partial);
   reduce_partials(partial, nblk, nvec, kNvMax, red, 0, nvec, nullptr, s);
   std::vector<double> Gr((size_t)nvec * kNvMax);

@@ -138,6 +138,10 @@ struct ApplyArgs {
   int nrhs;                // number of loads of the launch (set by the launchers)
 };
 
+namespace modal {
+int sm_count();   // SMs of the current device
+}
+
 // ---- modal element operators (modal.cuh, modal_f32.cu, modal_f64.cu) -----------
 struct DF {         // unevaluated pair h + l
   float h, l;
@@ -416,7 +420,7 @@ void copy_scale_f64(const double* r, double* v, i64 len, const double* sc, int n
 // Riesz representers in periodic H^1 (A = alpha^2 K + M, Chebyshev iteration
 // with exact spectral bounds), projection of the objective representer off
 // the constraint representers and the constraint correction; v (nn doubles).
-// work: 4 (1 + ncons) nn doubles; dptrs_dev: device room for 1 + ncons
+// work: 2 (1 + ncons) nn doubles; dptrs_dev: device room for 1 + ncons
 // pointers; partial / red as for reduce_partials; info (host, optional):
 // ||P g_J||_H, Chebyshev iterations, mu_1..mu_ncons.
 constexpr int kHilbertMaxCons = 8;
