@@ -16,14 +16,14 @@
 // all 304 products of the modal matrix the registers of a thread do not hold
 // the modes of an element.
 //
-// One warp owns a strip of RY node rows by 30 columns (lanes 1..30; lanes 0
-// and 31 are halo) and marches through z.  x neighbours are lane shuffles, y
-// neighbours the rows a thread holds, z neighbours registers carried from the
-// plane before: no shared memory, no barrier, no atomics, and every element
-// is evaluated once per strip (RY + 1 element rows for RY node rows).  The
-// columns of all strips form one sequence of nx + 2 positions per strip (both
-// periodic ends included), which warps cut into windows of 30 outputs, so any
-// nx keeps about 30/32 of the lanes busy.
+// A block owns a strip of node rows by 30 columns (lanes 1..30; lanes 0 and 31
+// are halo) and marches through z; its four warps take consecutive element rows.
+// x neighbours are lane shuffles, y neighbours the rows a thread holds (the row
+// between two warps goes through shared memory), z neighbours registers carried
+// from the plane before: no atomics, and 4 RE element rows serve 4 RE - 1 node
+// rows.  The columns of all strips form one sequence of nx + 2 positions per
+// strip (both periodic ends included), cut into windows of 30 outputs, so any nx
+// keeps about 30/32 of the lanes busy.
 #pragma once
 
 #include "kernels.cuh"
@@ -238,66 +238,76 @@ __device__ __forceinline__ void element(const typename MatOf<KIND, V>::type& K, 
 //   void fetch(pre, offset)     operands of a node's output
 //   void out(offset, acc, own, pre)   assembled values of the output components
 //                               and the node's own inputs
-template <int KIND, int RY, bool PF, typename V, typename IO>
-__device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, const IO& io, int nx, int ny, int nz,
-                                      int L) {
+//
+// Block = window of 30 columns (blockIdx.x) of a strip of 4 RE - 1 node rows,
+// warp w = the RE element rows from w RE.  Element row r of a warp lies between
+// its node rows r and r + 1; the node row 0 of a warp also needs the last
+// element row of the warp before, whose contribution comes through shared
+// memory (one barrier per plane, two buffers).  Warp 0's node row 0 is the halo.
+template <int KIND, typename V>
+struct Exchange {
+  Pair<V> p[2][kWarps][Shape<KIND>::NO][2][32];
+};
+
+template <int KIND, int RE, bool PF, typename V, typename IO>
+__device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, const IO& io, Exchange<KIND, V>& ex, int nx,
+                                      int ny, int nz, int L) {
   constexpr int NI = Shape<KIND>::NI, NO = Shape<KIND>::NO;
-  const int lane = threadIdx.x & 31;
+  constexpr int S = kWarps * RE - 1;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int rl = nx + 2;
-  const int strips = (ny + RY - 1) / RY;
-  const int p0 = (int)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * kOut;
-  if (p0 >= strips * rl - 2) return;   // warp-uniform
+  const int strips = (ny + S - 1) / S;
+  const int p0 = (int)blockIdx.x * kOut;
   const int p = min(p0 + lane, strips * rl - 1);
   const int strip = p / rl;
   const int xi = p - strip * rl - 1;
   const bool vx = lane >= 1 && lane <= kOut && p0 + lane == p && xi >= 0 && xi < nx;
   const int i = xi < 0 ? nx - 1 : (xi >= nx ? 0 : xi);
-  const int j0 = strip * RY;
-  // in-plane offsets of the node rows j0 - 1 .. j0 + RY (periodic); rows of
-  // the strip that this lane writes
-  unsigned ro[RY + 2];
-  bool ok[RY];
+  const int j0 = strip * S - 1 + w * RE;   // the warp's node row 0
+  // in-plane offsets of its node rows (periodic); rows that this lane writes
+  unsigned ro[RE + 1];
+  bool ok[RE];
+  {
+    int j = j0 < 0 ? j0 + ny : j0 % ny;
 #pragma unroll
-  for (int r = 0; r < RY + 2; ++r) {
-    int j = j0 - 1 + r;   // at most ny + RY - 1: two subtractions wrap it (RY <= 4, ny >= 2)
-    j = j < 0 ? j + ny : j;
-    j = j >= ny ? j - ny : j;
-    j = j >= ny ? j - ny : j;
-    ro[r] = (unsigned)(j * nx + i);
+    for (int r = 0; r < RE + 1; ++r) {
+      ro[r] = (unsigned)(j * nx + i);
+      j = j + 1 == ny ? 0 : j + 1;
+    }
   }
 #pragma unroll
-  for (int r = 0; r < RY; ++r) ok[r] = vx && j0 + r < ny;
+  for (int r = 0; r < RE; ++r) ok[r] = vx && j0 + r < ny && (r > 0 || w > 0);
   const unsigned nxy = (unsigned)(nx * ny);
   const int z0 = blockIdx.z * L;
   const int Lc = min(L, nz - z0);
-  Pair<V> ps[RY + 2][NI];   // x sums and differences of the plane before
-  V own[RY][NI];            // its values on the strip's own rows
-  Pair<V> carry[RY][NO];    // contributions of the layer below to the plane before
+  Pair<V> ps[RE + 1][NI];   // x sums and differences of the plane before
+  V own[RE][NI];            // its values
+  Pair<V> carry[RE][NO];    // contributions of the layer below to the plane before
   unsigned zp = (unsigned)(z0 == 0 ? nz - 1 : z0 - 1) * nxy;   // the plane before
-  unsigned zc = (unsigned)z0 * nxy;   // the plane above the layer
+  unsigned zc = (unsigned)z0 * nxy;                             // the plane above the layer
   // the loads of the first two planes are in flight together
-  V v0[RY + 2][NI], vn[PF ? RY + 2 : 1][NI], rn[PF ? RY + 1 : 1];
+  V v0[RE + 1][NI], vn[PF ? RE + 1 : 1][NI], rn[PF ? RE : 1];
 #pragma unroll
-  for (int r = 0; r < RY + 2; ++r)
+  for (int r = 0; r < RE + 1; ++r)
 #pragma unroll
     for (int d = 0; d < NI; ++d) v0[r][d] = io.in(d, zp + ro[r]);
   if (PF) {
 #pragma unroll
-    for (int r = 0; r < RY + 2; ++r)
+    for (int r = 0; r < RE + 1; ++r)
 #pragma unroll
       for (int d = 0; d < NI; ++d) vn[PF ? r : 0][d] = io.in(d, zc + ro[r]);
 #pragma unroll
-    for (int r = 0; r < RY + 1; ++r) rn[PF ? r : 0] = io.rho(zp + ro[r]);
+    for (int r = 0; r < RE; ++r) rn[PF ? r : 0] = io.rho(zp + ro[r]);
   }
 #pragma unroll
-  for (int r = 0; r < RY + 2; ++r)
+  for (int r = 0; r < RE + 1; ++r)
 #pragma unroll
     for (int d = 0; d < NI; ++d) {
-      const V w = vdown(v0[r][d]);
-      ps[r][d] = mk<V>(vadd(w, v0[r][d]), vsub(w, v0[r][d]));
+      const V u = vdown(v0[r][d]);
+      ps[r][d] = mk<V>(vadd(u, v0[r][d]), vsub(u, v0[r][d]));
     }
 #pragma unroll
-  for (int r = 0; r < RY; ++r) {
+  for (int r = 0; r < RE; ++r) {
 #pragma unroll
     for (int c = 0; c < NO; ++c) carry[r][c] = mk<V>(V{}, V{});
 #pragma unroll
@@ -306,42 +316,56 @@ __device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, co
 #pragma unroll 1
   for (int t = 0; t <= Lc; ++t) {
     const unsigned zn = zc + nxy == nxy * (unsigned)nz ? 0 : zc + nxy;
-    V v[RY + 2][NI], rho[RY + 1];
-    typename IO::Pre pre[RY];
+    V v[RE + 1][NI], rho[RE];
+    typename IO::Pre pre[RE];
     if (PF) {
 #pragma unroll
-      for (int r = 0; r < RY + 2; ++r)
+      for (int r = 0; r < RE + 1; ++r)
 #pragma unroll
         for (int d = 0; d < NI; ++d) {
           v[r][d] = vn[PF ? r : 0][d];
           vn[PF ? r : 0][d] = io.in(d, zn + ro[r]);
         }
 #pragma unroll
-      for (int r = 0; r < RY + 1; ++r) {
+      for (int r = 0; r < RE; ++r) {
         rho[r] = rn[PF ? r : 0];
         rn[PF ? r : 0] = io.rho(zc + ro[r]);
       }
     } else {
 #pragma unroll
-      for (int r = 0; r < RY + 2; ++r)
+      for (int r = 0; r < RE + 1; ++r)
 #pragma unroll
         for (int d = 0; d < NI; ++d) v[r][d] = io.in(d, zc + ro[r]);
 #pragma unroll
-      for (int r = 0; r < RY + 1; ++r) rho[r] = io.rho(zp + ro[r]);
+      for (int r = 0; r < RE; ++r) rho[r] = io.rho(zp + ro[r]);
     }
     if (t > 0) {
 #pragma unroll
-      for (int r = 0; r < RY; ++r)
-        if (ok[r]) io.fetch(pre[r], zp + ro[r + 1]);
+      for (int r = 0; r < RE; ++r)
+        if (ok[r]) io.fetch(pre[r], zp + ro[r]);
     }
-    Pair<V> q0[NI][2], up[NO][2];
+    // output row r from its element rows' contributions
+    auto emit = [&](int r, const Pair<V> (&up)[NO][2], const Pair<V> (&low)[NO][2]) {
+      V acc[NO];
 #pragma unroll
-    for (int r = 0; r < RY + 2; ++r) {
+      for (int c = 0; c < NO; ++c) {
+        const Pair<V> ts = padd(up[c][0], low[c][0]), td = padd(up[c][1], low[c][1]);
+        const Pair<V> o = padd(carry[r][c], psub(ts, td));
+        carry[r][c] = padd(ts, td);
+        acc[c] = vadd(vsub(sum_of(o), dif_of(o)), vup(vadd(sum_of(o), dif_of(o))));
+      }
+      if (t > 0 && ok[r]) io.out(zp + ro[r], acc, own[r], pre[r]);
+#pragma unroll
+      for (int d = 0; d < NI; ++d) own[r][d] = v[r][d];
+    };
+    Pair<V> q0[NI][2], up[NO][2], low0[NO][2];
+#pragma unroll
+    for (int r = 0; r < RE + 1; ++r) {
       Pair<V> q1[NI][2];
 #pragma unroll
       for (int d = 0; d < NI; ++d) {
-        const V w = vdown(v[r][d]);
-        const Pair<V> x = mk<V>(vadd(w, v[r][d]), vsub(w, v[r][d]));
+        const V u = vdown(v[r][d]);
+        const Pair<V> x = mk<V>(vadd(u, v[r][d]), vsub(u, v[r][d]));
         q1[d][0] = padd(x, ps[r][d]);
         q1[d][1] = psub(x, ps[r][d]);
         ps[r][d] = x;
@@ -349,18 +373,11 @@ __device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, co
       if (r > 0) {
         Pair<V> low[NO][2], un[NO][2];
         element<KIND, V>(K, q0, q1, rho[r - 1], low, un);
-        if (r > 1) {
-          V acc[NO];
+        if (r == 1) {
 #pragma unroll
-          for (int c = 0; c < NO; ++c) {
-            const Pair<V> ts = padd(up[c][0], low[c][0]), td = padd(up[c][1], low[c][1]);
-            const Pair<V> o = padd(carry[r - 2][c], psub(ts, td));
-            carry[r - 2][c] = padd(ts, td);
-            acc[c] = vadd(vsub(sum_of(o), dif_of(o)), vup(vadd(sum_of(o), dif_of(o))));
-          }
-          if (t > 0 && ok[r - 2]) io.out(zp + ro[r - 1], acc, own[r - 2], pre[r - 2]);
-#pragma unroll
-          for (int d = 0; d < NI; ++d) own[r - 2][d] = v[r - 1][d];
+          for (int c = 0; c < NO; ++c) low0[c][0] = low[c][0], low0[c][1] = low[c][1];
+        } else {
+          emit(r - 1, up, low);
         }
 #pragma unroll
         for (int c = 0; c < NO; ++c) up[c][0] = un[c][0], up[c][1] = un[c][1];
@@ -368,6 +385,17 @@ __device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, co
 #pragma unroll
       for (int d = 0; d < NI; ++d) q0[d][0] = q1[d][0], q0[d][1] = q1[d][1];
     }
+    // the last element row's upper contribution goes to the next warp
+#pragma unroll
+    for (int c = 0; c < NO; ++c)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) ex.p[t & 1][w][c][z][lane] = up[c][z];
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NO; ++c)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) up[c][z] = ex.p[t & 1][w == 0 ? 0 : w - 1][c][z][lane];
+    emit(0, up, low0);
     zp = zc;
     zc = zn;
   }
@@ -376,18 +404,18 @@ __device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, co
 // ---- launch geometry -----------------------------------------------------------
 int sm_count();   // modal_f32.cu
 
-// Planes per chunk: the smallest waves x (planes + 2) for the warps that the
+// Planes per chunk: the smallest waves x (planes + 2) for the blocks that the
 // chip holds (a chunk evaluates one element layer and loads two node planes
 // more than it writes).
-inline int chunk_planes(int nz, i64 warps, int warps_per_sm) {
-  const i64 slots = (i64)sm_count() * warps_per_sm;
+inline int chunk_planes(int nz, i64 blocks, int blocks_per_sm) {
+  const i64 slots = (i64)sm_count() * blocks_per_sm;
   int best = nz;
   const int most = nz < 4096 ? nz : 4096;   // grid z
   double cost = 1e300;
   for (int chunks = 1; chunks <= most; ++chunks) {
     const int L = (nz + chunks - 1) / chunks;
     if (chunks > 1 && L == (nz + chunks - 2) / (chunks - 1)) continue;
-    const i64 w = warps * ((nz + L - 1) / L);
+    const i64 w = blocks * ((nz + L - 1) / L);
     const double c = (double)((w + slots - 1) / slots) * (L + 2.0);
     if (c < cost) {
       cost = c;
@@ -397,13 +425,14 @@ inline int chunk_planes(int nz, i64 warps, int warps_per_sm) {
   return best;
 }
 
-// Grid (window groups, load groups, z chunks) and planes per chunk.
-inline dim3 grid_for(int nx, int ny, int nz, int groups, int rows, int blocks_per_sm, int* L) {
+// Grid (windows, load groups, z chunks) and planes per chunk, RE element rows
+// per warp.
+inline dim3 grid_for(int nx, int ny, int nz, int groups, int re, int blocks_per_sm, int* L) {
+  const int rows = kWarps * re - 1;
   const i64 seq = (i64)((ny + rows - 1) / rows) * (nx + 2) - 2;   // positions between the first and last halo
   const i64 windows = (seq + kOut - 1) / kOut;
-  const i64 blocks = (windows + kWarps - 1) / kWarps;
-  *L = chunk_planes(nz, blocks * kWarps * groups, blocks_per_sm * kWarps);
-  return dim3((unsigned)blocks, (unsigned)groups, (unsigned)((nz + *L - 1) / *L));
+  *L = chunk_planes(nz, windows * groups, blocks_per_sm);
+  return dim3((unsigned)windows, (unsigned)groups, (unsigned)((nz + *L - 1) / *L));
 }
 
 }  // namespace modal

@@ -32,10 +32,9 @@ struct DfIO {
   }
 };
 
-// Rows per strip at 128^3 / 64^3 / 32^3 with nine loads (us): one 3717 / 546 / 82,
-// two 3845 / 524 / 84 (4176 / 557 / 88 before the sums of the x pairs became
-// packed instructions; the corner form took 8300 at 128^3).  Both spill at 255
-// registers (184 and 560 bytes); the arithmetic alone would take about 1.5 ms.
+// Element rows per warp at 128^3 / 64^3 / 32^3 with nine loads (us): one 3746 / 478
+// / 74, two 4021 / 517 / 77 (the corner form took 8300 at 128^3).  Both spill at
+// 255 registers; the arithmetic alone would take about 1.5 ms.
 constexpr int kRows = 1, kBlocksPerSM = 2;
 
 __global__ void __launch_bounds__(modal::kThreads, kBlocksPerSM)
@@ -51,7 +50,8 @@ k_modal_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs, c
   io.b = b ? b + q * bs : nullptr;
   io.r = r + q * rs;
   io.nn = (i64)nx * ny * nz;
-  modal::march<MK_FULL, kRows, false, DF>(K, io, nx, ny, nz, L);
+  __shared__ modal::Exchange<MK_FULL, DF> ex;
+  modal::march<MK_FULL, kRows, false, DF>(K, io, ex, nx, ny, nz, L);
 }
 
 }  // namespace

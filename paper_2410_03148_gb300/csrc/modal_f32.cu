@@ -22,15 +22,17 @@ void modal_full<float>(const ModalArgs<float>& a, const ModalMat<float, 4, 4>& K
   modal::launch<MK_FULL, MM_APPLY, 3, 2, true, float>(a, K, s);
 }
 
-// Rows per strip and blocks per SM, measured with 9 loads at 128^3 / 64^3 / 16^3
-// (us).  Coupled operator: 3 rows, 2 blocks 321 / 53 / 8.2; 2 rows, 2 blocks
-// 341 / 55 / 8.2; 1 row, 3 blocks 521 / 72 / 8.2.  Elastic step: 3 rows, 2
-// blocks 290 / 47 / 6.3 (255 registers); 2 rows, 3 blocks 424 / 66 / 8.2 (spills
-// at 168 registers); 1 row, 4 blocks 384 / 60 / 6.3.  Sbar step: 2 rows, 6
-// blocks 113 / 18.7 / 6.1; 3 rows, 5 blocks 111 / 20.3; 4 rows, 5 blocks 177 /
-// 22.7 / 6.3.  Coupling: 4 rows, 4 blocks 143 / 24.6 / 6.3; 3 rows 153 / 22.8.
-// What is left: 128^3 runs at 60 % issue use with 8 warps per SM, 45 % of the
-// instructions are not arithmetic (addresses, constant loads, shuffles).
+// Element rows per warp (RE) and blocks per SM, measured with 9 loads at 128^3 /
+// 64^3 / 16^3 (us).  Coupled operator: RE 3, 2 blocks 265 / 45 / 6.3; RE 2, 3
+// blocks 291 / 47 / 6.3; RE 4, 2 blocks (no registers for the prefetch) 356 / 43.
+// Elastic step: RE 2, 3 blocks 282 / 46 / 6.2; RE 4, 2 blocks 291 / 45 / 6.3; RE 3,
+// 2 blocks 314 / 52; RE 1, 4 blocks 353 / 53.  Sbar step: RE 3, 6 blocks 111 /
+// 18.6 / 4.2; RE 2, 6 blocks 127 / 20.6; RE 4, 5 blocks 113 / 20.6 / 6.2.  Coupling:
+// RE 4, 4 blocks 125 / 20.6; RE 3, 4 blocks 196 / 25.  (Strips of single warps,
+// each with its own halo element row, took 318 / 51, 286 / 46, 113 / 18.5 and
+// 142 / 22.6.)  What is left: about 60 % issue use with 8 to 12 warps per SM, and
+// 45 % of the instructions are not arithmetic (addresses, constant loads,
+// shuffles); the elastic step's bytes alone would take 150 us at 128^3.
 template <>
 void modal_pu<float>(const ModalArgs<float>& a, const ModalMat<float, 1, 3>& K, int, cudaStream_t s) {
   modal::launch<MK_PU, MM_ADD, 4, 4, false, float>(a, K, s);
@@ -39,24 +41,24 @@ void modal_pu<float>(const ModalArgs<float>& a, const ModalMat<float, 1, 3>& K, 
 template <>
 void modal_uu<float>(const ModalArgs<float>& a, const ModalMat<float, 3, 3>& K, int mode, cudaStream_t s) {
   switch (mode) {
-    case MM_APPLY: modal::launch<MK_UU, MM_APPLY, 3, 2, true, float>(a, K, s); break;
-    case MM_RESID: modal::launch<MK_UU, MM_RESID, 3, 2, true, float>(a, K, s); break;
-    case MM_STEP: modal::launch<MK_UU, MM_STEP, 3, 2, true, float>(a, K, s); break;
-    case MM_STEP0: modal::launch<MK_UU, MM_STEP0, 3, 2, true, float>(a, K, s); break;
-    case MM_PRE: modal::launch<MK_UU, MM_PRE, 3, 2, true, float>(a, K, s); break;
-    default: modal::launch<MK_UU, MM_POST, 3, 2, true, float>(a, K, s); break;
+    case MM_APPLY: modal::launch<MK_UU, MM_APPLY, 2, 3, true, float>(a, K, s); break;
+    case MM_RESID: modal::launch<MK_UU, MM_RESID, 2, 3, true, float>(a, K, s); break;
+    case MM_STEP: modal::launch<MK_UU, MM_STEP, 2, 3, true, float>(a, K, s); break;
+    case MM_STEP0: modal::launch<MK_UU, MM_STEP0, 2, 3, true, float>(a, K, s); break;
+    case MM_PRE: modal::launch<MK_UU, MM_PRE, 2, 3, true, float>(a, K, s); break;
+    default: modal::launch<MK_UU, MM_POST, 2, 3, true, float>(a, K, s); break;
   }
 }
 
 template <>
 void modal_ss<float>(const ModalArgs<float>& a, const ModalSch<float>& K, int mode, cudaStream_t s) {
   switch (mode) {
-    case MM_APPLY: modal::launch<MK_SS, MM_APPLY, 2, 6, true, float>(a, K, s); break;
-    case MM_RESID: modal::launch<MK_SS, MM_RESID, 2, 6, true, float>(a, K, s); break;
-    case MM_STEP: modal::launch<MK_SS, MM_STEP, 2, 6, true, float>(a, K, s); break;
-    case MM_STEP0: modal::launch<MK_SS, MM_STEP0, 2, 6, true, float>(a, K, s); break;
-    case MM_PRE: modal::launch<MK_SS, MM_PRE, 2, 6, true, float>(a, K, s); break;
-    default: modal::launch<MK_SS, MM_POST, 2, 6, true, float>(a, K, s); break;
+    case MM_APPLY: modal::launch<MK_SS, MM_APPLY, 3, 6, true, float>(a, K, s); break;
+    case MM_RESID: modal::launch<MK_SS, MM_RESID, 3, 6, true, float>(a, K, s); break;
+    case MM_STEP: modal::launch<MK_SS, MM_STEP, 3, 6, true, float>(a, K, s); break;
+    case MM_STEP0: modal::launch<MK_SS, MM_STEP0, 3, 6, true, float>(a, K, s); break;
+    case MM_PRE: modal::launch<MK_SS, MM_PRE, 3, 6, true, float>(a, K, s); break;
+    default: modal::launch<MK_SS, MM_POST, 3, 6, true, float>(a, K, s); break;
   }
 }
 

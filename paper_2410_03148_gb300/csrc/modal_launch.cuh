@@ -65,9 +65,10 @@ struct IO {
   }
 };
 
-template <int KIND, int MODE, int RY, int MINB, bool PF, typename T>
+template <int KIND, int MODE, int RE, int MINB, bool PF, typename T>
 __global__ void __launch_bounds__(kThreads, MINB)
 k_modal(const ModalArgs<T> a, const __grid_constant__ typename MatOf<KIND, T>::type K, int L) {
+  __shared__ Exchange<KIND, T> ex;
   const int r1 = min(a.nrhs, ((int)blockIdx.y + 1) * a.rg);
 #pragma unroll 1
   for (int r = blockIdx.y * a.rg; r < r1; ++r) {
@@ -89,17 +90,18 @@ k_modal(const ModalArgs<T> a, const __grid_constant__ typename MatOf<KIND, T>::t
         if (MODE == MM_STEP0 || MODE == MM_PRE) io.k0[c] = *a.c0 * a.dk[c];
       }
     }
-    march<KIND, RY, PF, T>(K, io, a.nx, a.ny, a.nz, L);
+    if (r > (int)blockIdx.y * a.rg) __syncthreads();   // the buffers of the load before
+    march<KIND, RE, PF, T>(K, io, ex, a.nx, a.ny, a.nz, L);
   }
 }
 
-template <int KIND, int MODE, int RY, int MINB, bool PF, typename T>
+template <int KIND, int MODE, int RE, int MINB, bool PF, typename T>
 void launch(const ModalArgs<T>& a0, const typename MatOf<KIND, T>::type& K, cudaStream_t s) {
   ModalArgs<T> a = a0;
   if (a.rg < 1) a.rg = 1;
   int L = 0;
-  const dim3 grid = grid_for(a.nx, a.ny, a.nz, (a.nrhs + a.rg - 1) / a.rg, RY, MINB, &L);
-  note_launch(), k_modal<KIND, MODE, RY, MINB, PF, T><<<grid, kThreads, 0, s>>>(a, K, L);
+  const dim3 grid = grid_for(a.nx, a.ny, a.nz, (a.nrhs + a.rg - 1) / a.rg, RE, MINB, &L);
+  note_launch(), k_modal<KIND, MODE, RE, MINB, PF, T><<<grid, kThreads, 0, s>>>(a, K, L);
 }
 
 }  // namespace modal

@@ -1,9 +1,10 @@
 """GPU parity of the modal element operators (mm2 materials) and of the corner
 form that serves other materials, against the FP64 oracle, at the edges of the
-modal kernels' work split: warps own 30 columns of a sequence with nx + 2
-positions per strip of 2 to 4 node rows and march through chunks of z planes.
-Shapes (nz, ny, nx) cover rows that end a window or start one (nx = 28 .. 31,
-58 .. 61), rows shorter than a strip (ny = 2, 3), ragged last strips, the
+modal kernels' work split: blocks own 30 columns of a sequence with nx + 2
+positions per strip of 3, 7, 11 or 15 node rows (the four warps exchange the row
+between them) and march through chunks of z planes.  Shapes (nz, ny, nx) cover
+rows that end a window or start one (nx = 28 .. 31, 58 .. 61), rows shorter than
+a strip (ny = 2, 3), whole and ragged last strips (ny = 7, 11, 15, 16, 33), the
 smallest periodic sizes, several strips per window (small nx) and several
 chunks.  Tolerances: those of the oracle parity tests (FP64 1e-12, FP32 2e-6 of
 max|K| max|x| x 8; the FP32-pair residual 2e-14 of 8 x 32 terms), and for
@@ -39,7 +40,7 @@ def general_material():
 
 
 SHAPES = [(2, 2, 2), (3, 2, 28), (2, 3, 29), (3, 5, 30), (5, 4, 31), (2, 7, 58), (3, 6, 61), (9, 8, 3), (33, 9, 16),
-          (6, 33, 5), (4, 64, 64)]
+          (6, 33, 5), (3, 11, 9), (5, 15, 8), (4, 16, 30), (4, 64, 64), (40, 45, 50)]
 
 
 @pytest.mark.parametrize("shape,mat", [(s, "mm2") for s in SHAPES] + [(s, "general") for s in SHAPES[:3]])
