@@ -137,12 +137,13 @@ k_gs_dots(const T* __restrict__ V, i64 vstride, i64 len, int nv, double* __restr
 
 // w <- s (w - sum_{i<nb} c_i v_i), and the dots of the result with v_0 ..
 // v_{nb-1} and itself (index nb).  Up to R basis values per element stay in
-// registers between the two; more are read again, 16 at a time.
+// registers between the two (4, 8, 16, in FP32 also 24); more are read again,
+// 16 at a time.
 template <typename T, int R>
 __global__ void __launch_bounds__(kB)
 k_gs_update(T* __restrict__ V, i64 vstride, i64 len, int nb, const double* __restrict__ coef, double* __restrict__ partial,
             const int* __restrict__ active) {
-  constexpr int G = R <= 8 ? 8 : 16;
+  constexpr int G = R == 0 ? 16 : (R <= 8 ? 8 : (R <= 16 ? 16 : 32));
   __shared__ T sh[G * (kB + 1)];
   __shared__ T c[kNvMax + 1];
   const int q = blockIdx.y;
@@ -393,6 +394,8 @@ void gs_step(const GsArgs<T>& a, int j, cudaGraphConditionalHandle next, bool se
   if (nb <= 4) note_launch(), k_gs_update<T, 4><<<g, kB, 0, s>>>(a.V, a.vstride, a.len, nb, a.coef, a.partial, a.active);
   else if (nb <= 8) note_launch(), k_gs_update<T, 8><<<g, kB, 0, s>>>(a.V, a.vstride, a.len, nb, a.coef, a.partial, a.active);
   else if (nb <= 16) note_launch(), k_gs_update<T, 16><<<g, kB, 0, s>>>(a.V, a.vstride, a.len, nb, a.coef, a.partial, a.active);
+  else if (nb <= 24 && sizeof(T) == 4)
+    note_launch(), k_gs_update<T, sizeof(T) == 4 ? 24 : 0><<<g, kB, 0, s>>>(a.V, a.vstride, a.len, nb, a.coef, a.partial, a.active);
   else note_launch(), k_gs_update<T, 0><<<g, kB, 0, s>>>(a.V, a.vstride, a.len, nb, a.coef, a.partial, a.active);
   note_launch(), k_gs_finish<<<a.nrhs, kB, 0, s>>>(a.partial, a.nblk, j, a.m, a.gram, a.nu2, a.coef, a.hcol, a.H, a.cs,
                                                   a.sn, a.g, a.active, a.resid, a.tolabs, a.kcount, a.ticket,
