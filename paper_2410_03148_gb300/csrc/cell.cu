@@ -295,6 +295,7 @@ struct cell_handle {
   double *gram = nullptr, *nu2 = nullptr, *coef = nullptr, *gs_partial = nullptr;   // Gram-Schmidt (gs.cu)
   int gs_nblk = 1;
   int* ticket = nullptr;
+  int* sel = nullptr;        // selected loads (options.load_mask); the others' vectors stay zero
   double *resid = nullptr, *invscale = nullptr, *tolabs = nullptr, *ybuf = nullptr, *beta2 = nullptr;
   int *active = nullptr, *kcount = nullptr, *want = nullptr, *ranmask = nullptr;
   Krylov<float> kf;
@@ -972,13 +973,13 @@ cell::ModalArgs<T> modal_args(cell_handle* h, const T* x, i64 xs, T* y, i64 ys, 
 }
 
 // FP64-grade residual r = b - Ahat x of the split iterate (x = xh + xl)
-void residual_df(cell_handle* h, const double* b, double* r, int nrhs) {
+void residual_df(cell_handle* h, const double* b, double* r, int nrhs, const int* active) {
   const i64 len = 4 * h->nn;
   if (h->modal)
     cell::modal_resid_df(h->xh, h->xl, len, b, len, r, len, h->rho32, h->rho_l, h->mdf, h->nx, h->ny, h->nz, nrhs,
-                         h->st);
+                         active, h->st);
   else
-    cell::resid_df(h->xh, h->xl, len, b, len, r, len, h->rho32, h->rho_l, h->DF, h->nx, h->ny, h->nz, nrhs, nullptr,
+    cell::resid_df(h->xh, h->xl, len, b, len, r, len, h->rho32, h->rho_l, h->DF, h->nx, h->ny, h->nz, nrhs, active,
                    h->st);
 }
 
@@ -1403,6 +1404,12 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
   CKS(A.alloc(&h->coef, 9 * (kNvMax + 1)));
   h->gs_nblk = cell::gs_blocks(len);
   CKS(A.alloc(&h->gs_partial, (size_t)9 * kNvMax * h->gs_nblk));
+  CKS(A.alloc(&h->sel, 9));
+  {
+    int sel[9];
+    for (int q = 0; q < 9; ++q) sel[q] = (d->opt.load_mask >> q) & 1;
+    CK(cudaMemcpy(h->sel, sel, sizeof(sel), cudaMemcpyHostToDevice));
+  }
   CKS(A.alloc(&h->ticket, 1));
   CK(cudaMemsetAsync(h->ticket, 0, sizeof(int), h->st));
   CKS(A.alloc(&h->ybuf, 9 * kNvMax));
@@ -1570,9 +1577,9 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
       cell::gs_solution<T>(K.Z, 9 * len, len, h->ybuf, h->kcount, h->x64, h->xh, h->xl, 9, h->ranmask, s);
       cell::accum_iters(h->iters_d, h->kcount, h->ranmask, h->ctl_d, s);
       if constexpr (sizeof(T) == 4)
-        residual_df(h, h->b64, h->r64, 9);
+        residual_df(h, h->b64, h->r64, 9, h->sel);
       else
-        apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, nullptr, 9);
+        apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, h->sel, 9);
       cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
       cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->red, 0, 9, nullptr, s);
       cell::refine_ctl(h->bn2d, h->red, h->bfloor_d, P, h->want, h->tolabs, h->relres_d, h->iters_d, h->ctl_d, wh, s);
@@ -1732,10 +1739,10 @@ int solve_impl(cell_handle* h, cell_stats* st) {
     h->prof.cur_units = 9;
     if constexpr (sizeof(T) == 4) {
       const int ip = h->prof.begin(s, CELL_PROF_FULL64);
-      residual_df(h, h->b64, h->r64, 9);
+      residual_df(h, h->b64, h->r64, 9, h->sel);
       h->prof.end(CELL_PROF_FULL64, ip, s);
     } else {
-      apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, nullptr, 9);
+      apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, h->sel, 9);
     }
   }
   // null-space projection (mean displacement and potential per load)
@@ -2229,17 +2236,17 @@ int cell_homogenise(cell_handle* h, double CH[36], double eH[18], double kH[9]) 
   if (!h->solved || h->d.opt.load_mask != 0x1FF) return CELL_ESTATE;
   cudaStream_t s = h->st;
   const int nblk = h->nblk;
-  double G1[81], G2[81], srho;
+  double G[81], srho;
   cell::sum_reduce(h->rho64, h->nn, h->partial, nblk, h->red, s);
   CK(cudaMemcpyAsync(&srho, h->red, sizeof(double), cudaMemcpyDeviceToHost, s));
-  cell::gram9(h->b64, h->x64, h->nn, h->partial, nblk, h->red, s);
-  CK(cudaMemcpyAsync(G1, h->red, sizeof(G1), cudaMemcpyDeviceToHost, s));
-  cell::gram9(h->x64, h->r64, h->nn, h->partial, nblk, h->red2, s);
-  CK(cudaMemcpyAsync(G2, h->red2, sizeof(G2), cudaMemcpyDeviceToHost, s));
+  // b.y and y.r in one pass: the symmetric parts of sum y_I.r_J and of its
+  // transpose sum r_I.y_J are the same, and H is symmetrised below
+  cell::gram9(h->b64, h->x64, h->nn, h->partial, nblk, h->red2, s, h->r64);
+  CK(cudaMemcpyAsync(G, h->red2, sizeof(G), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   // energy form: H = sum rho H0e - b.y - y.r   (H0e = Zbar^T K0 Zbar)
   double H[81];
-  for (int i = 0; i < 81; ++i) H[i] = srho * h->H0e[i] - G1[i] - G2[i];
+  for (int i = 0; i < 81; ++i) H[i] = srho * h->H0e[i] - G[i];
   for (int I = 0; I < 9; ++I)
     for (int J = I + 1; J < 9; ++J) {
       const double v = 0.5 * (H[I * 9 + J] + H[J * 9 + I]);
@@ -2466,7 +2473,7 @@ int cell_apply(cell_handle* h, const void* x, void* y, int nrhs, int dtype) {
   } else if (dtype == CELL_F64_DF) {
     if (nrhs > 9) return CELL_EINVAL;
     cell::split_f64(static_cast<const double*>(x), h->xh, h->xl, (i64)nrhs * len, h->st);
-    residual_df(h, nullptr, static_cast<double*>(y), nrhs);
+    residual_df(h, nullptr, static_cast<double*>(y), nrhs, nullptr);
   } else {
     return CELL_EINVAL;
   }

@@ -101,31 +101,29 @@ k_rhs9(const double* __restrict__ rho, const __grid_constant__ RhsParams P, int 
   const i64 n = (i64)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= nn) return;
   const int i = (int)(n % nx), j = (int)((n / nx) % ny), k = (int)(n / nxy);
-  double acc[4][9];
-#pragma unroll
-  for (int c = 0; c < 4; ++c)
-#pragma unroll
-    for (int I = 0; I < 9; ++I) acc[c][I] = 0.0;
+  double r[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
-    const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2;
-    const int la = (1 - ex) + 2 * (1 - ey) + 4 * (1 - ez);
-    const int ei = ex ? i : (i == 0 ? nx - 1 : i - 1);
-    const int ej = ey ? j : (j == 0 ? ny - 1 : j - 1);
-    const int ek = ez ? k : (k == 0 ? nz - 1 : k - 1);
-    const double r = rho[ei + nx * (ej + (i64)ny * ek)];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int I = 0; I < 9; ++I) acc[c][I] = fma(r, P.F[(4 * la + c) * 9 + I], acc[c][I]);
+    const int ei = (e & 1) ? i : (i == 0 ? nx - 1 : i - 1);
+    const int ej = ((e >> 1) & 1) ? j : (j == 0 ? ny - 1 : j - 1);
+    const int ek = (e >> 2) ? k : (k == 0 ? nz - 1 : k - 1);
+    r[e] = rho[ei + nx * (ej + (i64)ny * ek)];
   }
+  // the products of a load that is not selected are not formed (FP64 rate)
 #pragma unroll
-  for (int I = 0; I < 9; ++I)
+  for (int I = 0; I < 9; ++I) {
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    if ((mask >> I) & 1) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const double v = ((mask >> I) & 1) ? (c == 3 ? acc[c][I] : -acc[c][I]) : 0.0;
-      b[((i64)I * 4 + c) * nn + n] = v;
+      for (int e = 0; e < 8; ++e) {
+        const int la = 7 - e;   // local index of the node in the element at (ex, ey, ez)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[c] = fma(r[e], P.F[(4 * la + c) * 9 + I], acc[c]);
+      }
     }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) b[((i64)I * 4 + c) * nn + n] = ((mask >> I) & 1) ? (c == 3 ? acc[c] : -acc[c]) : 0.0;
+  }
 }
 
 // grid (nblk, nrhs*4): partial sums of each (rhs, comp) plane.
@@ -150,9 +148,9 @@ __global__ void k_sub_means(double* __restrict__ x, i64 nn, const double* __rest
     X[k] -= m;
 }
 
-// grid (nblk, 9): row I of sum_c sgn_c <u^I_c, v^J_c>, J = 0..8.
+// grid (nblk, 9): row I of sum_c sgn_c <u^I_c + t^I_c, v^J_c>, J = 0..8 (t optional).
 __global__ void __launch_bounds__(kB)
-k_gram9(const double* __restrict__ u, const double* __restrict__ v, i64 nn,
+k_gram9(const double* __restrict__ u, const double* __restrict__ t, const double* __restrict__ v, i64 nn,
         double* __restrict__ partial) {
   __shared__ double sh[kWarps];
   const int I = blockIdx.y;
@@ -165,7 +163,7 @@ k_gram9(const double* __restrict__ u, const double* __restrict__ v, i64 nn,
   for (int J = 0; J < 9; ++J) acc[J] = 0.0;
   for (i64 k = lo + threadIdx.x; k < hi; k += kB) {
     const double sg = (k >= 3 * nn) ? -1.0 : 1.0;
-    const double uk = sg * U[k];
+    const double uk = sg * (t ? U[k] + t[(i64)I * len + k] : U[k]);
 #pragma unroll
     for (int J = 0; J < 9; ++J) acc[J] = fma(uk, v[(i64)J * len + k], acc[J]);
   }
@@ -501,8 +499,8 @@ void sub_means(double* x, i64 nn, int nrhs, const double* sums, cudaStream_t s) 
 }
 
 void gram9(const double* u, const double* v, i64 nn, double* partial, int nblk, double* out,
-           cudaStream_t s) {
-  note_launch(), k_gram9<<<dim3(nblk, 9), kB, 0, s>>>(u, v, nn, partial);
+           cudaStream_t s, const double* t) {
+  note_launch(), k_gram9<<<dim3(nblk, 9), kB, 0, s>>>(u, t, v, nn, partial);
   reduce_partials(partial, nblk, 9, 9, out, 0, 9, nullptr, s);
 }
 

@@ -204,7 +204,7 @@ template <typename T> void modal_ss(const ModalArgs<T>& a, const ModalSch<T>& K,
 // FP64-grade r = b - Ahat x (r = Ahat x if b is null) in pairs of FP32, as resid_df
 void modal_resid_df(const float* xh, const float* xl, i64 xs, const double* b, i64 bs, double* r, i64 rs,
                     const float* rho_h, const float* rho_l, const ModalMat<DF, 4, 4>& K, int nx, int ny, int nz,
-                    int nrhs, cudaStream_t s);
+                    int nrhs, const int* active, cudaStream_t s);
 
 // Constant-bank slots holding (K0, S0) in FP32 for the fixed-matrix kernels;
 // returns slot + 1, or 0 if none is free.  Release with cslot_release.
@@ -452,9 +452,9 @@ void rhs9(const double* rho, const RhsParams& F, int mask, double* b, int nx, in
 void comp_sums(const double* x, i64 nn, int nrhs, double* partial, int nblk, double* out,
                cudaStream_t s);
 void sub_means(double* x, i64 nn, int nrhs, const double* sums, cudaStream_t s);
-// G_IJ (+)= sum_n sum_c sgn_c u^I_c v^J_c, sgn = -1 for the potential component
+// G_IJ = sum_n sum_c sgn_c (u + t)^I_c v^J_c, sgn = -1 for the potential component, t optional
 void gram9(const double* u, const double* v, i64 nn, double* partial, int nblk, double* out,
-           cudaStream_t s);
+           cudaStream_t s, const double* t = nullptr);
 // out[0] = sum of x[0..n) (or of the squares)  (device scalar)
 void sum_reduce(const double* x, i64 n, double* partial, int nblk, double* out, cudaStream_t s,
                 int squares = 0);

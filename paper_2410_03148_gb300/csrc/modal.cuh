@@ -412,15 +412,15 @@ inline int chunk_planes(int nz, i64 blocks, int blocks_per_sm) {
   int best = nz;
   const int most = nz < 4096 ? nz : 4096;   // grid z
   double cost = 1e300;
-  for (int chunks = 1; chunks <= most; ++chunks) {
+  for (int chunks = 1; chunks <= most;) {
     const int L = (nz + chunks - 1) / chunks;
-    if (chunks > 1 && L == (nz + chunks - 2) / (chunks - 1)) continue;
     const i64 w = blocks * ((nz + L - 1) / L);
     const double c = (double)((w + slots - 1) / slots) * (L + 2.0);
     if (c < cost) {
       cost = c;
       best = L;
     }
+    chunks = L > 1 ? (nz + L - 2) / (L - 1) : most + 1;   // the next count with shorter chunks
   }
   return best;
 }

@@ -40,8 +40,9 @@ constexpr int kRows = 1, kBlocksPerSM = 2;
 __global__ void __launch_bounds__(modal::kThreads, kBlocksPerSM)
 k_modal_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs, const double* __restrict__ b, i64 bs,
            double* __restrict__ r, i64 rs, const float* __restrict__ rho_h, const float* __restrict__ rho_l,
-           const __grid_constant__ ModalMat<DF, 4, 4> K, int nx, int ny, int nz, int L) {
+           const __grid_constant__ ModalMat<DF, 4, 4> K, int nx, int ny, int nz, const int* active, int L) {
   const int q = blockIdx.y;
+  if (active && !__any_sync(0xffffffffu, active[q])) return;
   DfIO io;
   io.xh = xh + q * xs;
   io.xl = xl + q * xs;
@@ -58,10 +59,10 @@ k_modal_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs, c
 
 void modal_resid_df(const float* xh, const float* xl, i64 xs, const double* b, i64 bs, double* r, i64 rs,
                     const float* rho_h, const float* rho_l, const ModalMat<DF, 4, 4>& K, int nx, int ny, int nz,
-                    int nrhs, cudaStream_t s) {
+                    int nrhs, const int* active, cudaStream_t s) {
   int L = 0;
   const dim3 grid = modal::grid_for(nx, ny, nz, nrhs, kRows, kBlocksPerSM, &L);
-  note_launch(), k_modal_df<<<grid, modal::kThreads, 0, s>>>(xh, xl, xs, b, bs, r, rs, rho_h, rho_l, K, nx, ny, nz, L);
+  note_launch(), k_modal_df<<<grid, modal::kThreads, 0, s>>>(xh, xl, xs, b, bs, r, rs, rho_h, rho_l, K, nx, ny, nz, active, L);
 }
 
 }  // namespace cell
