@@ -344,6 +344,12 @@ __device__ __forceinline__ void march(const typename MatOf<KIND, V>::type& K, co
       for (int r = 0; r < RE; ++r)
         if (ok[r]) io.fetch(pre[r], zp + ro[r]);
     }
+    // tall strips of few warps: the next plane's operands come from DRAM to L2
+    // meanwhile (Sbar step at 128^3 102 -> 93 us; no gain with more warps per SM)
+    if (RE >= 6) {
+#pragma unroll
+      for (int r = 0; r < RE; ++r) io.prefetch(zc + ro[r]);
+    }
     // output row r from its element rows' contributions
     auto emit = [&](int r, const Pair<V> (&up)[NO][2], const Pair<V> (&low)[NO][2]) {
       V acc[NO];

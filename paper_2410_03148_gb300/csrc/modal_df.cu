@@ -22,6 +22,7 @@ struct DfIO {
 #pragma unroll
     for (int c = 0; c < 4; ++c) p.b[c] = b ? __ldg(b + c * nn + o) : 0.0;
   }
+  __device__ __forceinline__ void prefetch(unsigned) const {}
   __device__ __forceinline__ void out(unsigned o, DF (&acc)[4], const DF (&)[4], const Pre& p) const {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {

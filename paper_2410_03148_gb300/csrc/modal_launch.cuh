@@ -42,6 +42,14 @@ struct IO {
       if (kXp) p.xp[c] = xp[c * nn + o];
     }
   }
+  __device__ __forceinline__ static void l2(const T* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+  __device__ __forceinline__ void prefetch(unsigned o) const {
+#pragma unroll
+    for (int c = 0; c < NO; ++c) {
+      if (kB && MODE != MM_PRE) l2(b + c * nn + o);
+      if (kXp) l2(xp + c * nn + o);
+    }
+  }
   __device__ __forceinline__ void out(unsigned o, T (&acc)[NO], const T (&own)[NI], const Pre& p) const {
     if (KIND == MK_FULL) acc[NO - 1] = -acc[NO - 1];
 #pragma unroll

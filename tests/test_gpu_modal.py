@@ -83,6 +83,22 @@ def test_operators_match_oracle(shape, mat):
                 assert err < 2e-14 * 8 * 32 * kmax * np.abs(x).max(), (nrhs, err)
 
 
+def test_large_grid_sbar_matches_fp64():
+    """Sbar in FP32 above the size from which a warp takes six element rows (23
+    node rows per strip, ragged here), against the FP64 kernel (FP32 bound
+    2e-6 of max|S0| max|x| x 8)."""
+    from paper_2410_03148_gb300 import Cell
+    from paper_2410_03148_gb300 import _binding as B
+    M = cellgen.pzt5h_class()
+    shape = (77, 85, 91)
+    cell = Cell(torch.as_tensor(cellgen.random_rho(shape, seed=5), device="cuda:0"), M, kind="rho", autotune=0, restart=1)
+    x = torch.randn((9, 1) + shape, device="cuda:0", dtype=torch.float32, generator=torch.Generator("cuda:0").manual_seed(1))
+    y = cell.apply_block("Sbar", x).double()
+    want = cell.apply_block("Sbar", x.double())
+    S0 = B.cell_element_matrices(cell._desc)[1]
+    assert float((y - want).abs().max()) < 2e-6 * 8 * np.abs(S0).max() * float(x.abs().max())
+
+
 @pytest.mark.parametrize("shape", [(6, 7, 5), (8, 8, 8)])
 @pytest.mark.parametrize("precision", [0, 1])
 def test_general_material_solve_matches_oracle(shape, precision):
