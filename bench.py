@@ -57,11 +57,18 @@ CLASS_COST = {
     "schur0": (2 * (64 + 8), 4 * (1 + 2 + 2 + 1) + 4 / 9 + 4 / 9, "hbm", "f32", 1),
     "coupling": (2 * (192 + 8), 4 * (3 + 1 + 1) + 4 / 9, "alu", "f32", 3),
 }
-# The tensor-core smoothers (node-centric TF32 MMAs): each (node, load) row
-# takes 15 MMAs of K = 8 against N = 32 columns, 2 x 120 x 32 flops; their
-# algorithmic bytes are those of the class above, which bound them (the MMA
-# work at the TF32 rate takes less time than the bytes at the HBM rate).
-TC_FLOPS_PER_ROW = 2 * 120 * 32
+# Materials with the mm2 mirror planes (the bench's) run the modal operators: the
+# same with their operation counts and the bytes of the three-term Chebyshev
+# steps, averaged over the six launches of a V-cycle (first steps from b alone: 6
+# floats per component-triple read and written; second step, residual and first
+# post-smoothing step 9; two full steps 12).
+MODAL_COST = {
+    "full32": (2 * 82 + 156, 4 * 4 + 4 * 4 + 4 / 9, "hbm", "f32", 4),
+    "full64": (8 * (2 * 82 + 156), 8 * 4 + 8 * 4 + 8 * 4 + 8 / 9, "alu", "f32", 4),
+    "elastic0": (2 * 45 + 117, 4 * (6 + 3 * 9 + 2 * 12) / 6 + 2 * 4 / 9, "hbm", "f32", 3),
+    "schur0": (7 + 39, 4 * (2 + 3 * 3 + 2 * 4) / 6 + 2 * 4 / 9, "hbm", "f32", 1),
+    "coupling": (2 * 15 + 65, 4 * (3 + 1 + 1) + 4 / 9, "hbm", "f32", 3),
+}
 # Algorithmic bytes per dof and load of the plain FP32 operator apply
 # (read x, write y, rho amortised over 4 dof x 9 loads)
 APPLY_BYTES_PER_DOF_RHS = 4 + 4 + 4 / 36
@@ -91,7 +98,7 @@ def parse():
     ap.add_argument("--inner-tol", type=float, default=1e-4)
     ap.add_argument("--no-accuracy", action="store_true")
     ap.add_argument("--accuracy-designs", type=int, default=2)
-    # fine-grid smoothers on the tensor cores (node-centric tcgen05 TF32 kernels)
+    # cell_options.tensor_cores (2: the Krylov operator on the tensor cores)
     ap.add_argument("--tensor-cores", type=int, default=1, choices=[0, 1, 2])
     # E1 benchmark of the paper's weak-scaling study instead of the headline step
     ap.add_argument("--e1", action="store_true")
@@ -135,14 +142,6 @@ def peaks():
             d = json.load(f)
         return d.get("hbm_gbs", 6800.0), "measured", d.get("sm_max_mhz", 2070.0)
     return 6800.0, "fallback", 2070.0
-
-
-def peaks_tf32():
-    p = os.path.join(ROOT, "MEASURED_PEAKS.json")
-    if os.path.exists(p):
-        with open(p) as f:
-            return json.load(f).get("bf16_tflops", 1900.0) / 2.0
-    return 1900.0 / 2.0
 
 
 class ClockSampler:
@@ -493,10 +492,7 @@ def main():
     tot = {c: sum(s["class_ms"][c] for s in stats) for c in B.PROF_CLASSES}
     cnt = {c: sum(s["class_count"][c] for s in stats) for c in B.PROF_CLASSES}
     units = {c: sum(s["class_units"][c] for s in stats) for c in B.PROF_CLASSES}
-    flops_u, bytes_u, bound, kdt, ndof = CLASS_COST[dom]
-    tc_class = args.tensor_cores >= 1 and prec == 1 and dom in ("elastic0", "schur0")
-    if tc_class:
-        bound = "hbm"
+    flops_u, bytes_u, bound, kdt, ndof = (MODAL_COST if prec == 1 else CLASS_COST)[dom]
     nn = n ** 3
     avg_ms = tot[dom] / max(cnt[dom], 1)
     per_launch_units = units[dom] / max(cnt[dom], 1)
@@ -517,14 +513,6 @@ def main():
         roof["traffic"] = tt["bytes_per_node_load"] * nn * per_launch_units
         roof["traffic_source"] = (f"ncu dram__bytes_read+write of one {tt.get('n')}^3 launch "
                                   f"({tt.get('profile')}), per node and load, scaled to this launch")
-    if tc_class:
-        # tensor-pipe view: MMA flops per launch (the Schur kernel packs four loads per row)
-        rows = nn * per_launch_units / (4 if dom == "schur0" else 1)
-        tf32_peak = peaks_tf32()
-        roof["tensor_view"] = {"mma_tflops": TC_FLOPS_PER_ROW * rows / (avg_ms * 1e-3) / 1e12,
-                               "tf32_peak_tflops": tf32_peak,
-                               "frac": TC_FLOPS_PER_ROW * rows / (avg_ms * 1e-3) / 1e12 / tf32_peak,
-                               "peak_source": "measured bf16 burst (MEASURED_PEAKS.json) / 2, the nominal TF32 ratio"}
     dof_rate = ndof * nn * per_launch_units / (avg_ms * 1e-3)
     roof.update({"kernel": dom,
                  "peak_source": (f"hbm {hbm_kind} (MEASURED_PEAKS.json)" if bound == "hbm" else

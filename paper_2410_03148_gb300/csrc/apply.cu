@@ -330,76 +330,6 @@ k_apply_fixed_ld(const ApplyArgs<T> a, const __grid_constant__ FixedMat<T, NCM> 
   epilogue<T, NCO, MODE>(a, r, t, acc, dold);
 }
 
-// Per-element (Galerkin) matrices on a coarse level.  One thread per node
-// and group of RG loads (grid z = 9 / RG groups): each element row block
-// (NC x 8NC values, entry-major in memory so a warp's loads coalesce) is read
-// once per group and applied to the group's loads.  Large levels use RG = 3
-// (fewer matrix reads), small levels RG = 1 (more parallelism).
-template <typename T, int NC, int RG, int MODE>
-__global__ void __launch_bounds__(kBlock) k_apply_elem(const ApplyArgs<T> a, int nrhs) {
-  NodeIdx t;
-  if (!node_index(a.nx, a.ny, a.nz, t)) return;
-  const int r0 = blockIdx.z * RG;
-  bool on[RG];
-  bool any = false;
-#pragma unroll
-  for (int g = 0; g < RG; ++g) {
-    on[g] = (r0 + g < nrhs) && !(a.active && !a.active[r0 + g]);
-    any = any || on[g];
-  }
-  if (!any) return;
-  const i64 ne = t.nn;
-  constexpr int R = 8 * NC;
-  T acc[RG][NC];
-#pragma unroll
-  for (int g = 0; g < RG; ++g)
-#pragma unroll
-    for (int c = 0; c < NC; ++c) acc[g][c] = T(0);
-#pragma unroll 1
-  for (int e = 0; e < 8; ++e) {
-    const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2;
-    const int la = (1 - ex) + 2 * (1 - ey) + 4 * (1 - ez);
-    // neighbour offsets of this element's corners, by select (no local arrays)
-    const i64 x0 = ex ? t.xo[1] : t.xo[0], x1 = ex ? t.xo[2] : t.xo[1];
-    const i64 y0 = ey ? t.yo[1] : t.yo[0], y1 = ey ? t.yo[2] : t.yo[1];
-    const i64 z0 = ez ? t.zo[1] : t.zo[0], z1 = ez ? t.zo[2] : t.zo[1];
-    const i64 el = x0 + y0 + z0;
-    const T* K = a.ke + (i64)(la * NC) * R * ne + el;
-    T km[NC][R];
-#pragma unroll
-    for (int c = 0; c < NC; ++c)
-#pragma unroll
-      for (int b = 0; b < R; ++b) km[c][b] = __ldg(K + (i64)(c * R + b) * ne);
-    int m[8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b)
-      m[b] = (int)(((b & 1) ? x1 : x0) + (((b >> 1) & 1) ? y1 : y0) + ((b >> 2) ? z1 : z0));
-#pragma unroll
-    for (int g = 0; g < RG; ++g) {
-      if (!on[g]) continue;
-      const T* X = a.x + (r0 + g) * a.xs;
-#pragma unroll
-      for (int b = 0; b < 8; ++b)
-#pragma unroll
-        for (int d = 0; d < NC; ++d) {
-          const T xv = __ldg(X + d * t.nn + m[b]);
-#pragma unroll
-          for (int c = 0; c < NC; ++c) acc[g][c] = fma(km[c][b * NC + d], xv, acc[g][c]);
-        }
-    }
-  }
-#pragma unroll
-  for (int g = 0; g < RG; ++g) {
-    if (!on[g]) continue;
-    const int r = r0 + g;
-    T dold[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c)
-      dold[c] = (MODE == AM_CHEB || MODE == AM_CHEB_LAST) ? a.x[r * a.xs + c * t.nn + t.n] : T(0);
-    epilogue<T, NC, MODE>(a, r, t, acc[g], dold);
-  }
-}
-
 // Assembled block stencil on a coarse level: y_n = sum_q S_n[q] x_{n+q} over the
 // 27 neighbours q (offsets in {-1,0,1}^3, q = dx + 3 dy + 9 dz).  One thread per
 // node and group of RG loads; the node's stencil row (27 NC x NC blocks) is
@@ -718,24 +648,6 @@ void apply_ss(const ApplyArgs<T>& a, const FixedMat<T, 1>& M, int mode, int nrhs
 }
 
 template <typename T, int NC, int RG>
-void launch_elem(const ApplyArgs<T>& a, int mode, int nrhs, cudaStream_t s) {
-  const dim3 g = grid_for(a, (nrhs + RG - 1) / RG);
-  switch (mode) {
-    case AM_LINEAR: note_launch(), k_apply_elem<T, NC, RG, AM_LINEAR><<<g, kBlock, 0, s>>>(a, nrhs); break;
-    case AM_CHEB: note_launch(), k_apply_elem<T, NC, RG, AM_CHEB><<<g, kBlock, 0, s>>>(a, nrhs); break;
-    case AM_CHEB_LAST: note_launch(), k_apply_elem<T, NC, RG, AM_CHEB_LAST><<<g, kBlock, 0, s>>>(a, nrhs); break;
-    default: note_launch(), k_apply_elem<T, NC, RG, AM_RESID_CHEB0><<<g, kBlock, 0, s>>>(a, nrhs); break;
-  }
-}
-
-template <typename T, int NC>
-void apply_elem(const ApplyArgs<T>& a, int mode, int nrhs, cudaStream_t s) {
-  const long long nn = (long long)a.nx * a.ny * a.nz;
-  if (nn >= 16384) launch_elem<T, NC, 3>(a, mode, nrhs, s);
-  else launch_elem<T, NC, 1>(a, mode, nrhs, s);
-}
-
-template <typename T, int NC, int RG>
 void launch_st(const ApplyArgs<T>& a, int mode, int nrhs, cudaStream_t s) {
   const dim3 g0 = grid_for(a, (nrhs + RG - 1) / RG);
   const dim3 g(g0.z, g0.x, g0.y);   // load groups fastest (see k_apply_st)
@@ -896,8 +808,6 @@ void cslot_release(int slot1) {
   template void apply_uu<T>(const ApplyArgs<T>&, const FixedMat<T, 4>&, int, int, cudaStream_t);   \
   template void apply_pu<T>(const ApplyArgs<T>&, const FixedMat<T, 4>&, int, cudaStream_t);        \
   template void apply_ss<T>(const ApplyArgs<T>&, const FixedMat<T, 1>&, int, int, cudaStream_t);   \
-  template void apply_elem<T, 1>(const ApplyArgs<T>&, int, int, cudaStream_t);                     \
-  template void apply_elem<T, 3>(const ApplyArgs<T>&, int, int, cudaStream_t);                     \
   template void apply_stencil<T, 1>(const ApplyArgs<T>&, int, int, cudaStream_t, int);             \
   template void apply_stencil<T, 3>(const ApplyArgs<T>&, int, int, cudaStream_t, int);             \
   template int stencil_autotune<T, 1>(const ApplyArgs<T>&, int, int, cudaStream_t, float*);        \

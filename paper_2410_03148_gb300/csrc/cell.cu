@@ -1426,7 +1426,8 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
     float k0f[1024], s0f[64];
     for (int i = 0; i < 1024; ++i) k0f[i] = (float)h->K0[i];
     for (int i = 0; i < 64; ++i) s0f[i] = (float)h->S0[i];
-    if (d->opt.const_bank) h->cslot1 = cell::cslot_acquire(k0f, s0f);
+    // (the modal operators of mm2 materials do not read the slots)
+    if (d->opt.const_bank && !h->modal) h->cslot1 = cell::cslot_acquire(k0f, s0f);
     CKS(setup_krylov<float>(h));
   } else {
     CKS(setup_krylov<double>(h));

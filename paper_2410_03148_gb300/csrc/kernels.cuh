@@ -127,7 +127,6 @@ struct ApplyArgs {
   T* dout; i64 ds;         // CHEB / RESID_CHEB0: new search direction
   const T* dinv;           // [NC][nn] inverse diagonal
   const T* rho;            // per-element scale (fixed-matrix operators)
-  const T* ke;             // per-element matrices, SoA: ke[entry*ne + e]
   const T* st;             // assembled 27-point block stencil, SoA: st[((q*NC+c)*NC+d)*nn + n]
   T alpha, beta, c1, c2;
   const T* cc;             // if set: device (c1, c2) pair used instead of c1, c2
@@ -224,9 +223,6 @@ template <typename T> void apply_pu(const ApplyArgs<T>& a, const FixedMat<T, 4>&
 // Local-Schur operator Sbar = sum rho_e S0 (1 -> 1).
 template <typename T> void apply_ss(const ApplyArgs<T>& a, const FixedMat<T, 1>& M, int mode,
                                     int nrhs, cudaStream_t s);
-// Per-element-matrix operator on a coarse level (NC = 1 or 3).
-template <typename T, int NC> void apply_elem(const ApplyArgs<T>& a, int mode, int nrhs,
-                                              cudaStream_t s);
 // Assembled-stencil operator on a coarse level (NC = 1 or 3), a.st set; rg =
 // loads per thread (1, 3 or 9; 0 = size heuristic), bitwise-neutral.
 template <typename T, int NC> void apply_stencil(const ApplyArgs<T>& a, int mode, int nrhs,
