@@ -9,8 +9,9 @@
 // the matrix sits in a __constant__ slot (or, when all slots are taken, in a
 // by-value kernel parameter), so every multiply-add reads its coefficient
 // straight from the constant bank; the full operator pairs its multiply-adds
-// (two FP32 FMAs per instruction).  Coarse multigrid levels carry one Galerkin
-// matrix per element, stored entry-major (coalesced), or an assembled stencil.
+// (two FP32 FMAs per instruction).  Galerkin levels carry an assembled 27-point
+// stencil.  Materials with the mm2 mirror planes use the modal operators
+// (modal.cuh) instead.
 //
 // Operator definitions: Eq. (sym-piezo) and its nonsymmetric second form
 // (potential rows negated), §2.5; block operators of P_SCP, §2.5.3.

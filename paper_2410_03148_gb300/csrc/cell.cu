@@ -1121,7 +1121,7 @@ int gmres_cycle(cell_handle* h, const double* tolabs_host, int* iters) {
   cudaStream_t s = h->st;
   const int nblk = h->nblk;
   // beta^2 = |r|^2
-  cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, h->want, s);
+  cell::dot<double>(h->r64, len, h->r64, len, len, h->partial, nblk, kNvMax, 9, h->want, s);
   cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->beta2, 0, 9, h->want, s);
   CK(cudaMemcpyAsync(h->tolabs, tolabs_host, 9 * sizeof(double), cudaMemcpyHostToDevice, s));
   cell::start_cycle(h->beta2, h->g, h->nu2, m, h->active, h->want, h->resid, h->invscale, h->tolabs, h->kcount, 9, s);
@@ -1538,7 +1538,7 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
       cudaMemsetAsync(h->x64, 0, 9 * len * sizeof(double), s);
       cudaMemsetAsync(h->xh, 0, 9 * len * sizeof(float), s);
       cudaMemsetAsync(h->xl, 0, 9 * len * sizeof(float), s);
-      cell::multidot<double>(h->b64, 0, len, 1, h->b64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
+      cell::dot<double>(h->b64, len, h->b64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
       cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->bn2d, 0, 9, nullptr, s);
       cudaMemcpyAsync(h->r64, h->b64, 9 * len * sizeof(double), cudaMemcpyDeviceToDevice, s);
       cell::ctl_reset(h->ctl_d, h->iters_d, s);
@@ -1561,7 +1561,7 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
   if (e == cudaSuccess)
     e = capture_into(h, wbody, [&]() -> cudaError_t {
       cudaStream_t s = h->st;
-      cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, h->want, s);
+      cell::dot<double>(h->r64, len, h->r64, len, len, h->partial, nblk, kNvMax, 9, h->want, s);
       cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->beta2, 0, 9, h->want, s);
       cell::start_cycle(h->beta2, h->g, h->nu2, m, h->active, h->want, h->resid, h->invscale, h->tolabs, h->kcount, 9, s);
       cell::cycle_handles(h->active, h->ranmask, IH, s);
@@ -1581,7 +1581,7 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
         residual_df(h, h->b64, h->r64, 9, h->sel);
       else
         apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, h->sel, 9);
-      cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
+      cell::dot<double>(h->r64, len, h->r64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
       cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->red, 0, 9, nullptr, s);
       cell::refine_ctl(h->bn2d, h->red, h->bfloor_d, P, h->want, h->tolabs, h->relres_d, h->iters_d, h->ctl_d, wh, s);
       h->seg_ce = cell::g_launches.load() - nb;
@@ -1700,7 +1700,7 @@ int solve_impl(cell_handle* h, cell_stats* st) {
   CK(cudaMemsetAsync(h->xh, 0, 9 * len * sizeof(float), s));
   CK(cudaMemsetAsync(h->xl, 0, 9 * len * sizeof(float), s));
   double bn2[9], rn2[9];
-  cell::multidot<double>(h->b64, 0, len, 1, h->b64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
+  cell::dot<double>(h->b64, len, h->b64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
   cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->red, 0, 9, nullptr, s);
   std::vector<double> tmp(9 * kNvMax);
   CK(cudaMemcpyAsync(tmp.data(), h->red, 9 * kNvMax * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1710,7 +1710,7 @@ int solve_impl(cell_handle* h, cell_stats* st) {
   int status = CELL_OK;
   int refine = 0;
   while (true) {
-    cell::multidot<double>(h->r64, 0, len, 1, h->r64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
+    cell::dot<double>(h->r64, len, h->r64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
     cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->red, 0, 9, nullptr, s);
     CK(cudaMemcpyAsync(tmp.data(), h->red, 9 * kNvMax * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

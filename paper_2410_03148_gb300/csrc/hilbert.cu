@@ -12,7 +12,7 @@
 // extremes (corners of the cosine box) bound the spectrum exactly and the
 // iteration count for a given reduction follows in advance.  The objective and
 // constraint representers are solved together (one launch per step, one
-// vector per grid z slice).
+// vector per grid y index).
 //
 // Projection (null-space method): with the H Gram matrix G_ab = <g_a, g_b>_H
 // = g_a . d_b, the constraint block factors as R^T R (R = the Gram-Schmidt

@@ -351,10 +351,9 @@ template <typename T> void dense_solve(const T* Ainv, int n, const T* b, i64 bs,
                                        i64 nn, int nc, int nrhs, const int* active, cudaStream_t s);
 
 // ---- Krylov helpers (krylov.cu) ---------------------------------------------
-// partial[(q*nblk + blk)*nvmax + i] = block-partial of <V_i, w> for rhs q.
-template <typename T> void multidot(const T* V, i64 vstride, i64 rstride, int nv, const T* w,
-                                    i64 wstride, i64 len, double* partial, int nblk, int nvmax,
-                                    int nrhs, const int* active, cudaStream_t s);
+// partial[(q*nblk + blk)*nvmax] = block-partial of <v, w> for rhs q.
+template <typename T> void dot(const T* v, i64 vstride, const T* w, i64 wstride, i64 len, double* partial, int nblk,
+                               int nvmax, int nrhs, const int* active, cudaStream_t s);
 // out[q*nvmax + i] (+)= sum over blocks of partial
 void reduce_partials(const double* partial, int nblk, int nv, int nvmax, double* out, int accumulate,
                      int nrhs, const int* active, cudaStream_t s);

@@ -58,41 +58,27 @@ __device__ __forceinline__ void block_sum_many(double (&v)[G], double (*sh)[G]) 
   }
 }
 
-constexpr int kGrp = 8;
-
-// grid (nblk, nrhs, ceil(nv / G)); each block computes the partial dots of w
-// with the G basis vectors of its group over a contiguous chunk of len.  The
-// element loop is unrolled so that each thread keeps several elements' loads
-// in flight (these kernels are bound by HBM latency and bandwidth).
-template <typename T, int G>
+// grid (nblk, nrhs): each block computes the partial dot of v and w over a
+// contiguous chunk of len.  The loop is unrolled so that each thread keeps
+// several elements' loads in flight (bound by HBM latency and bandwidth).
+template <typename T>
 __global__ void __launch_bounds__(kB)
-k_multidot(const T* __restrict__ V, i64 vstride, i64 rstride, int nv, const T* __restrict__ w,
-           i64 wstride, i64 len, double* __restrict__ partial, int nvmax, const int* active) {
-  __shared__ double sh[kWarps][G];
+k_dot(const T* __restrict__ v, i64 vstride, const T* __restrict__ w, i64 wstride, i64 len,
+      double* __restrict__ partial, int nvmax, const int* active) {
+  __shared__ double sh[kWarps][1];
   const int q = blockIdx.y;
   if (active && !active[q]) return;
-  const int g0 = blockIdx.z * G;
-  const int ng = nv - g0 < G ? nv - g0 : G;
   const i64 chunk = (len + gridDim.x - 1) / gridDim.x;
   const i64 lo = (i64)blockIdx.x * chunk;
   const i64 hi = lo + chunk < len ? lo + chunk : len;
   const T* W = w + q * wstride;
-  const T* V0 = V + q * rstride + (i64)g0 * vstride;
-  T acc[G];
-#pragma unroll
-  for (int i = 0; i < G; ++i) acc[i] = T(0);
+  const T* V = v + q * vstride;
+  T acc = T(0);
 #pragma unroll 2
-  for (i64 k = lo + threadIdx.x; k < hi; k += kB) {
-    const T wk = W[k];
-#pragma unroll
-    for (int i = 0; i < G; ++i)
-      if (i < ng) acc[i] = fma(V0[(i64)i * vstride + k], wk, acc[i]);
-  }
-  double d[G];
-#pragma unroll
-  for (int i = 0; i < G; ++i) d[i] = (double)acc[i];
-  block_sum_many<G>(d, sh);
-  if (threadIdx.x < ng) partial[((i64)q * gridDim.x + blockIdx.x) * nvmax + g0 + threadIdx.x] = d[0];
+  for (i64 k = lo + threadIdx.x; k < hi; k += kB) acc = fma(V[k], W[k], acc);
+  double d[1] = {(double)acc};
+  block_sum_many<1>(d, sh);
+  if (threadIdx.x == 0) partial[((i64)q * gridDim.x + blockIdx.x) * nvmax] = d[0];
 }
 
 // One warp per (rhs, i): fixed-order sum over blocks.
@@ -164,17 +150,9 @@ inline unsigned stream_blocks(i64 len) {
 }  // namespace
 
 template <typename T>
-void multidot(const T* V, i64 vstride, i64 rstride, int nv, const T* w, i64 wstride, i64 len,
-              double* partial, int nblk, int nvmax, int nrhs, const int* active, cudaStream_t s) {
-  // one vector (norms): a single accumulator; else groups of 8
-  if (nv == 1) {
-    note_launch(), k_multidot<T, 1><<<dim3(nblk, nrhs, 1), kB, 0, s>>>(V, vstride, rstride, nv, w, wstride,
-                                                                       len, partial, nvmax, active);
-    return;
-  }
-  const unsigned ng = (unsigned)((nv + kGrp - 1) / kGrp);
-  note_launch(), k_multidot<T, kGrp><<<dim3(nblk, nrhs, ng), kB, 0, s>>>(V, vstride, rstride, nv, w, wstride,
-                                                                         len, partial, nvmax, active);
+void dot(const T* v, i64 vstride, const T* w, i64 wstride, i64 len, double* partial, int nblk, int nvmax, int nrhs,
+         const int* active, cudaStream_t s) {
+  note_launch(), k_dot<T><<<dim3(nblk, nrhs), kB, 0, s>>>(v, vstride, w, wstride, len, partial, nvmax, active);
 }
 
 void reduce_partials(const double* partial, int nblk, int nv, int nvmax, double* out, int accumulate,
@@ -200,7 +178,7 @@ void to_f32_scaled(const double* r, i64 rs, float* v, i64 vs, i64 len, const dou
   note_launch(), k_to_f32<<<dim3(stream_blocks(len), nrhs), kB, 0, s>>>(r, rs, v, vs, len, sc, active);
 }
 
-template void multidot<double>(const double*, i64, i64, int, const double*, i64, i64, double*, int, int, int,
-                               const int*, cudaStream_t);
+template void dot<double>(const double*, i64, const double*, i64, i64, double*, int, int, int, const int*,
+                          cudaStream_t);
 
 }  // namespace cell
