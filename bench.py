@@ -642,7 +642,7 @@ def main():
                        "refinements": [s["refinements"] for s in stats],
                        "tc_tiles_autotuned": {"elastic": stats[0]["tc_tiles"][0], "schur": stats[0]["tc_tiles"][1]},
                        "class_ms_per_step": share_ms, "class_share": class_share,
-                       "class_source": "separate fully profiled pass over the same designs "
+                       "class_source": "separate fully profiled pass over the first two designs "
                                        "(untimed); the timed region times only the roofline kernel"},
         }
         print(json.dumps(line), flush=True)
