@@ -769,7 +769,7 @@ std::mutex g_slot_mu;
 SlotState g_slots[64][kSlots];
 }  // namespace
 
-int cslot_acquire(const float* K0f, const float* S0f) {
+int cslot_acquire(const float* K0f, const float* S0f, cudaStream_t s) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   std::lock_guard<std::mutex> lk(g_slot_mu);
@@ -783,8 +783,12 @@ int cslot_acquire(const float* K0f, const float* S0f) {
   for (int i = 0; i < kSlots; ++i) {
     SlotState& st = g_slots[dev][i];
     if (st.refs == 0) {
-      if (cudaMemcpyToSymbol(c_k0, K0f, 1024 * sizeof(float), (size_t)i * 1024 * sizeof(float)) != cudaSuccess ||
-          cudaMemcpyToSymbol(c_s0, S0f, 64 * sizeof(float), (size_t)i * 64 * sizeof(float)) != cudaSuccess)
+      // done before the lock is released: handles on other streams may share the slot
+      if (cudaMemcpyToSymbolAsync(c_k0, K0f, 1024 * sizeof(float), (size_t)i * 1024 * sizeof(float),
+                                  cudaMemcpyHostToDevice, s) != cudaSuccess ||
+          cudaMemcpyToSymbolAsync(c_s0, S0f, 64 * sizeof(float), (size_t)i * 64 * sizeof(float),
+                                  cudaMemcpyHostToDevice, s) != cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess)
         return 0;
       std::memcpy(st.k0, K0f, sizeof(st.k0));
       std::memcpy(st.s0, S0f, sizeof(st.s0));

@@ -385,6 +385,15 @@ void fill_modal_set(const double* Km, const double* Sm, ModalSet<T>& M) {
   for (int m = 0; m < 8; ++m) M.ss.s[m] = (T)Sm[m * 8 + m];
 }
 
+// Host table to the device at set-up, ordered on the handle's stream (which may
+// not wait for the legacy default stream); the host copy is free on return.
+template <typename T>
+int upload(cell_handle* h, T* dst, const T* src, size_t n) {
+  CK(cudaMemcpyAsync(dst, src, n * sizeof(T), cudaMemcpyHostToDevice, h->st));
+  CK(cudaStreamSynchronize(h->st));
+  return CELL_OK;
+}
+
 template <typename T> const T* rho_of(cell_handle* h);
 template <> const float* rho_of<float>(cell_handle* h) { return h->rho32; }
 template <> const double* rho_of<double>(cell_handle* h) { return h->rho64; }
@@ -501,7 +510,7 @@ int alloc_mg(cell_handle* h, BlockMG<T>& mg, const double* fixed_block) {
               G[(size_t)c * R * R + (A * NC + d) * R + B * NC + e] = (T)v;
             }
     CKS(h->arena.alloc(&mg.childm, (size_t)8 * R * R));
-    CK(cudaMemcpy(mg.childm, G.data(), G.size() * sizeof(T), cudaMemcpyHostToDevice));
+    CKS(upload(h, mg.childm, G.data(), G.size()));
   }
   mg.lv.clear();
   Level<T> L0;
@@ -803,7 +812,7 @@ int alloc_mg_modal(cell_handle* h, BlockMG<T>& mg) {
     if (cell::dense_invert_ok((int)nd)) {
       CKS(h->arena.alloc(&mg.dwork, cell::dense_invert_work((int)nd)));
       CKS(h->arena.alloc(&mg.dk, R * R));
-      CK(cudaMemcpy(mg.dk, Lc.kb.data(), R * R * sizeof(double), cudaMemcpyHostToDevice));
+      CKS(upload(h, mg.dk, Lc.kb.data(), R * R));
     }
   }
   // Chebyshev coefficients (the bounds do not depend on the design): (0, 1 / theta),
@@ -1366,8 +1375,8 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
     unsigned short* dgf;
     CKS(A.alloc(&dbf, bf.size()));
     CKS(A.alloc(&dgf, gf.size()));
-    CK(cudaMemcpy(dbf, bf.data(), bf.size() * sizeof(float), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(dgf, gf.data(), gf.size() * 2, cudaMemcpyHostToDevice));
+    CKS(upload(h, dbf, bf.data(), bf.size()));
+    CKS(upload(h, dgf, gf.data(), gf.size()));
     h->tct.b_full = dbf;
     h->tct.g_full = dgf;
   }
@@ -1379,7 +1388,7 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
     cell::nc_build_b(cell::NK_UU, h->K0, h->S0, tb.data());
     cell::nc_build_b(cell::NK_SS4, h->K0, h->S0, tb.data() + nt);
     CKS(A.alloc(&h->ncb, tb.size()));
-    CK(cudaMemcpy(h->ncb, tb.data(), tb.size() * sizeof(float), cudaMemcpyHostToDevice));
+    CKS(upload(h, h->ncb, tb.data(), tb.size()));
   }
   for (int i = 0; i < 1024; ++i) h->kf.K0.k[i] = (float)h->K0[i];
   h->kd.rho = h->rho64;
@@ -1408,7 +1417,7 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
   {
     int sel[9];
     for (int q = 0; q < 9; ++q) sel[q] = (d->opt.load_mask >> q) & 1;
-    CK(cudaMemcpy(h->sel, sel, sizeof(sel), cudaMemcpyHostToDevice));
+    CKS(upload(h, h->sel, sel, 9));
   }
   CKS(A.alloc(&h->ticket, 1));
   CK(cudaMemsetAsync(h->ticket, 0, sizeof(int), h->st));
@@ -1427,7 +1436,7 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
     for (int i = 0; i < 1024; ++i) k0f[i] = (float)h->K0[i];
     for (int i = 0; i < 64; ++i) s0f[i] = (float)h->S0[i];
     // (the modal operators of mm2 materials do not read the slots)
-    if (d->opt.const_bank && !h->modal) h->cslot1 = cell::cslot_acquire(k0f, s0f);
+    if (d->opt.const_bank && !h->modal) h->cslot1 = cell::cslot_acquire(k0f, s0f, h->st);
     CKS(setup_krylov<float>(h));
   } else {
     CKS(setup_krylov<double>(h));

@@ -207,7 +207,7 @@ void modal_resid_df(const float* xh, const float* xl, i64 xs, const double* b, i
 
 // Constant-bank slots holding (K0, S0) in FP32 for the fixed-matrix kernels;
 // returns slot + 1, or 0 if none is free.  Release with cslot_release.
-int cslot_acquire(const float* K0f, const float* S0f);
+int cslot_acquire(const float* K0f, const float* S0f, cudaStream_t s);
 void cslot_release(int slot1);
 
 // ---- operator applies (apply.cu) -------------------------------------------
