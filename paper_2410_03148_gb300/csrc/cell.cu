@@ -867,8 +867,8 @@ int fill_mg_modal(cell_handle* h) {
 template <typename T>
 int finish_mg_modal(cell_handle* h, const unsigned dev[2]) {
   Krylov<T>& K = kry<T>(h);
-  if (K.mgu.dwork && cell::dense_invert_failed(dev[0])) CKS((dense_inverse<T, 3>(h, K.mgu)));
-  if (K.mgp.dwork && cell::dense_invert_failed(dev[1])) CKS((dense_inverse<T, 1>(h, K.mgp)));
+  if (K.mgu.dwork && cell::dense_invert_failed(dev[0], sizeof(T) == 8)) CKS((dense_inverse<T, 3>(h, K.mgu)));
+  if (K.mgp.dwork && cell::dense_invert_failed(dev[1], sizeof(T) == 8)) CKS((dense_inverse<T, 1>(h, K.mgp)));
   return CELL_OK;
 }
 

@@ -15,7 +15,12 @@ namespace {
 
 constexpr int kTile = 7;                 // register tile of a thread: kTile x kTile
 constexpr int kMaxN = 32 * kTile;        // 224 unknowns
-constexpr double kAccept = 1e-3;         // max |I - A X| before the last Newton step
+// Largest max |I - A X| before the last Newton step whose result is kept.  The
+// step leaves (I - A X)^2, entries of at most n times the square: 2^-53 for an
+// FP64 inverse, 2^-26 for one that is stored in FP32.  Designs reach 1e-12 at
+// contrasts of 1e-3 and about 1e-9 at 1e-8; beyond, the host factorises in FP64.
+constexpr double kAccept64 = 7e-10, kAccept32 = 8e-6;
+static_assert(kMaxN * kAccept64 * kAccept64 < 1.2e-16 && kMaxN * kAccept32 * kAccept32 < 1.5e-8, "accepted residual");
 
 // Row (i, c) of A = sum_e rho_e P_e^T K P_e: block = row, thread = column.  On
 // 2-node axes a node is several corners of one element: all matches count.
@@ -179,11 +184,11 @@ k_dense_mul(const double* __restrict__ A, const double* __restrict__ B, double* 
 
 bool dense_invert_ok(int n) { return n <= kMaxN; }
 size_t dense_invert_work(int n) { return (size_t)4 * n * n; }
-bool dense_invert_failed(unsigned dev_bits) {
+bool dense_invert_failed(unsigned dev_bits, bool fp64) {
   float f;
   static_assert(sizeof(f) == sizeof(dev_bits), "float bits");
   __builtin_memcpy(&f, &dev_bits, 4);
-  return !(f <= kAccept);
+  return !(f <= (fp64 ? kAccept64 : kAccept32));
 }
 
 template <typename T>

@@ -311,10 +311,10 @@ template <typename T, int NC> void mg_scale(const T* b, i64 bs, T* x, i64 xs, co
 // dense_invert_ok: out = (sum_e rho_e P_e^T K P_e + regularisation)^-1; K:
 // device, (8 nc)^2 FP64; work: dense_invert_work(n) doubles; *dev receives the
 // float bits of the residual before the last correction, to be judged with
-// dense_invert_failed.
+// dense_invert_failed (fp64: out is FP64).
 bool dense_invert_ok(int n);
 size_t dense_invert_work(int n);
-bool dense_invert_failed(unsigned dev_bits);
+bool dense_invert_failed(unsigned dev_bits, bool fp64);
 template <typename T> void dense_invert(const T* rho, const double* K, int nc, int nx, int ny, int nz, double* work,
                                         T* out, unsigned* dev, cudaStream_t s);
 

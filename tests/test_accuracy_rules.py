@@ -1,0 +1,32 @@
+"""Host rules that bound the rounding errors of the solver's kernels (no GPU):
+called in the built library by their C++ names."""
+import ctypes
+import os
+import struct
+
+import pytest
+
+LIB = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2410_03148_gb300", "libcell.so")
+
+
+@pytest.fixture(scope="module")
+def lib():
+    if not os.path.exists(LIB):
+        from paper_2410_03148_gb300 import build
+        build.build()
+    return ctypes.CDLL(LIB)
+
+
+def test_coarsest_inverse_is_kept_only_at_its_own_precision(lib):
+    """Newton-Schulz leaves the square of the residual R before its last step,
+    entries of at most n max|R|^2 with n <= 224 unknowns: an inverse is kept if
+    that is below FP64 rounding (2^-52), or FP32 rounding (2^-24) where it is
+    stored in FP32, and never with a residual that is no number."""
+    failed = lib._ZN4cell19dense_invert_failedEjb
+    failed.argtypes, failed.restype = (ctypes.c_uint, ctypes.c_bool), ctypes.c_bool
+    bits = lambda v: struct.unpack("I", struct.pack("f", v))[0]
+    for fp64, eps in ((True, 2.0 ** -52), (False, 2.0 ** -24)):
+        edge = (eps / 224) ** 0.5
+        assert failed(bits(1.01 * edge), fp64)
+        assert failed(bits(float("nan")), fp64) and failed(bits(float("inf")), fp64)
+        assert not failed(bits(0.2 * edge), fp64) and not failed(0, fp64)
