@@ -30,3 +30,16 @@ def test_coarsest_inverse_is_kept_only_at_its_own_precision(lib):
         assert failed(bits(1.01 * edge), fp64)
         assert failed(bits(float("nan")), fp64) and failed(bits(float("inf")), fp64)
         assert not failed(bits(0.2 * edge), fp64) and not failed(0, fp64)
+
+
+def test_gram_schmidt_chains_are_short(lib):
+    """A thread of the Gram-Schmidt dots chains FP32 products before its value
+    enters the block's compensated sum: at most 32 until a load has 1024 blocks
+    of 256 threads, the fewest blocks of a load's other reductions."""
+    blocks = lib._ZN4cell9gs_blocksEx
+    blocks.argtypes, blocks.restype = (ctypes.c_longlong,), ctypes.c_int
+    for n in list(range(2, 130)) + [160, 192, 256, 400, 736]:
+        length = 4 * n ** 3
+        b = blocks(length)
+        assert 1 <= b <= 1024
+        assert b >= min(1024, -(-length // (32 * 256))), n
