@@ -49,7 +49,8 @@ METRIC = "cell-solve time to C^H at 1e-8 rel err; DOF·RHS/s per apply vs HBM ro
 
 # Algorithmic cost per (node, load) of each timed kernel class of the library:
 # (flops, bytes, bound, dtype, dof per node).  Bytes count one read of every
-# input and one write of every output.
+# input and one write of every output.  Corner form (other materials than the
+# bench's):
 CLASS_COST = {
     "full32": (2 * (1024 + 32), 4 * 4 + 4 * 4 + 4 / 9, "alu", "f32", 4),
     "full64": (2 * (1024 + 32), 8 * 4 + 8 * 4 + 8 + 8 / 9, "alu", "f64", 4),
@@ -69,6 +70,19 @@ MODAL_COST = {
     "schur0": (7 + 39, 4 * (2 + 3 * 3 + 2 * 4) / 6 + 2 * 4 / 9, "hbm", "f32", 1),
     "coupling": (2 * 15 + 65, 4 * (3 + 1 + 1) + 4 / 9, "hbm", "f32", 3),
 }
+
+
+def class_cost(cls, prec):
+    """Cost entry of a kernel class of the bench's (mm2) solves, prec 1: mixed,
+    0: FP64.  FP64 solves run the same modal operators on operands of 8 bytes;
+    FP64 arithmetic (1/64 rate) bounds them, and full64 is the native operator
+    of the Arnoldi steps instead of the residual in FP32 pairs."""
+    if prec == 1:
+        return MODAL_COST[cls]
+    flops, nbytes, _, _, ndof = MODAL_COST["full32" if cls == "full64" else cls]
+    return flops, 2 * nbytes, "alu", "f64", ndof
+
+
 # Algorithmic bytes per dof and load of the plain FP32 operator apply
 # (read x, write y, rho amortised over 4 dof x 9 loads)
 APPLY_BYTES_PER_DOF_RHS = 4 + 4 + 4 / 36
@@ -455,7 +469,7 @@ def main():
     # class shares from a fully profiled pass over the timed designs (untimed)
     shares = [step(designs[k % ndes], profile=1)[0] for k in range(min(args.steps, 2))]
     share_ms = {c: sum(s_["class_ms"][c] for s_ in shares) / len(shares) for c in B.PROF_CLASSES}
-    dom = max((c for c in CLASS_COST), key=lambda c: share_ms[c])
+    dom = max((c for c in MODAL_COST), key=lambda c: share_ms[c])
     cells[2] = Cell(designs[0], mat, kind="phi", precision=prec, profile=1,
                     profile_mask=1 << B.PROF_CLASSES.index(dom), **sopt)
     step(designs[0], profile=2)
@@ -492,7 +506,7 @@ def main():
     tot = {c: sum(s["class_ms"][c] for s in stats) for c in B.PROF_CLASSES}
     cnt = {c: sum(s["class_count"][c] for s in stats) for c in B.PROF_CLASSES}
     units = {c: sum(s["class_units"][c] for s in stats) for c in B.PROF_CLASSES}
-    flops_u, bytes_u, bound, kdt, ndof = (MODAL_COST if prec == 1 else CLASS_COST)[dom]
+    flops_u, bytes_u, bound, kdt, ndof = class_cost(dom, prec)
     nn = n ** 3
     avg_ms = tot[dom] / max(cnt[dom], 1)
     per_launch_units = units[dom] / max(cnt[dom], 1)
@@ -508,22 +522,24 @@ def main():
         peak = fp32_peak if kdt == "f32" else fp64_peak
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": None}
-    tt = traffic_table().get(dom)
+    tt = traffic_table().get(dom) if prec == 1 else None   # (captures of the FP32 kernels)
     if tt and tt.get("bytes_per_node_load"):
         roof["traffic"] = tt["bytes_per_node_load"] * nn * per_launch_units
         roof["traffic_source"] = (f"ncu dram__bytes_read+write of one {tt.get('n')}^3 launch "
                                   f"({tt.get('profile')}), per node and load, scaled to this launch")
     dof_rate = ndof * nn * per_launch_units / (avg_ms * 1e-3)
+    apply_rate = hbm * 1e9 / (APPLY_BYTES_PER_DOF_RHS * (1 if prec == 1 else 2))
     roof.update({"kernel": dom,
                  "peak_source": (f"hbm {hbm_kind} (MEASURED_PEAKS.json)" if bound == "hbm" else
-                                 f"{nsm} SMs x 128 FP32 lanes x 2 x {sm_max:.0f} MHz"),
+                                 f"{nsm} SMs x 128 FP32 lanes x 2 x {sm_max:.0f} MHz" if kdt == "f32" else
+                                 "1.25 TFLOP/s FP64 (nominal)"),
                  "launches": cnt[dom], "avg_launch_ms": avg_ms, "loads_per_launch": per_launch_units,
                  "algorithmic_bytes_per_launch": alg_bytes,
                  "hbm_frac_of_algorithmic_bytes": alg_bytes / (avg_ms * 1e-3) / 1e9 / hbm,
                  "dof_per_node": ndof,
                  "dof_rhs_per_s": dof_rate,
-                 "dof_rhs_per_s_apply_roofline": hbm * 1e9 / APPLY_BYTES_PER_DOF_RHS,
-                 "dof_rhs_per_s_frac_of_apply_roofline": dof_rate / (hbm * 1e9 / APPLY_BYTES_PER_DOF_RHS)})
+                 "dof_rhs_per_s_apply_roofline": apply_rate,
+                 "dof_rhs_per_s_frac_of_apply_roofline": dof_rate / apply_rate})
     step_avg = total_ms / args.steps
     class_share = {c: round(share_ms[c] / max(step_avg, 1e-9), 4) for c in B.PROF_CLASSES}
 
