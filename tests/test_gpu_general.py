@@ -24,7 +24,8 @@ import pytest
 import torch
 
 import cellgen
-from oracle import ersatz, fem
+from oracle import ersatz, fem, laminate, precond, sensitivity
+from oracle.material import nondimensionalise
 
 pytestmark = pytest.mark.gpu
 
@@ -69,8 +70,11 @@ def close(a, b, tol):
 @functools.lru_cache(maxsize=None)
 def oracle_16():
     phi = cellgen.gaussian_levelset(16, seed=1)
-    ref = fem.solve_cell(ersatz.rho_from_levelset(phi), *material())
-    return phi, tuple(ref[k] for k in ("C", "e", "kappa"))
+    return phi, fem.solve_cell(ersatz.rho_from_levelset(phi), *material())
+
+
+def tensors(ref):
+    return tuple(ref[k] for k in ("C", "e", "kappa"))
 
 
 @pytest.mark.parametrize("opt", [{"tensor_cores": 0}, {"tensor_cores": 1}, {"tensor_cores": 2}, {"graphs": 0},
@@ -80,7 +84,89 @@ def test_solve_with_a_stencil_level_matches_oracle(opt):
     phi, ref = oracle_16()
     st, out = solved(phi, **opt)
     assert st["nlevels_u"] == 3
-    assert close(out, ref, 1e-8), st
+    assert close(out, tensors(ref), 1e-8), st
+
+
+@pytest.mark.parametrize("shape", [(16, 16, 16), (3, 17, 23), (7, 31, 24), (40, 16, 32)])
+def test_operators_match_oracle(shape):
+    """Corner-form operators over several blocks of a plane (the last one
+    ragged), FP64, FP32 and FP32 pairs, nine loads; tolerances of the oracle
+    parity tests."""
+    from paper_2410_03148_gb300 import Cell
+    from paper_2410_03148_gb300 import _binding as B
+    M = material()
+    rho = cellgen.random_rho(shape, seed=21)
+    cell = Cell(torch.as_tensor(rho, device="cuda:0"), M, kind="rho", autotune=0, restart=2)
+    N = rho.size
+    P = fem.CellProblem(rho, *M)
+    Cn, en, kn, _ = nondimensionalise(*M)
+    K0 = fem.element_matrix(Cn, en, kn, fem.cell_h(shape))
+    full, sign = P.Kg.tocsr().astype(float), np.tile([1.0, 1.0, 1.0, -1.0], N)[:, None]
+    ops = [("full", 4, lambda v: sign * (full @ v), np.abs(K0).max())]
+    for blk, nc in (("A", 3), ("Sbar", 1)):
+        Ke = precond.block_matrix(K0, blk)
+        A = precond.assemble_block(rho, Ke, nc, shape)
+        ops.append((blk, nc, lambda v, A=A: A @ v, np.abs(Ke).max()))
+    x = np.random.default_rng(22).standard_normal((9, 4) + shape)
+    for name, nc, mul, kmax in ops:
+        v = x[:, :nc]
+        for dt, tol in ((torch.float64, 1e-12), (torch.float32, 2e-6), ("pairs", 32 * 2e-14)):
+            if dt == "pairs" and name != "full":
+                continue
+            xt = torch.as_tensor(np.ascontiguousarray(v), device="cuda:0", dtype=torch.float64 if dt == "pairs" else dt)
+            if dt == "pairs":
+                y = torch.empty_like(xt)
+                B.cell_apply(cell._h, xt.data_ptr(), y.data_ptr(), 9, B.CELL_F64_DF)
+            else:
+                y = cell.apply(xt) if name == "full" else cell.apply_block(name, xt)
+            xd = xt.double().cpu().numpy().reshape(9, nc, N).transpose(2, 1, 0).reshape(-1, 9)
+            want = mul(xd).reshape(N, nc, 9).transpose(2, 1, 0).reshape(v.shape)
+            err = np.abs(y.double().cpu().numpy() - want).max()
+            assert err < tol * 8 * kmax * np.abs(v).max(), (name, dt, err)
+
+
+@pytest.mark.parametrize("gdtype,tol", [(torch.float64, 1e-8), (torch.float32, 1e-5)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_sensitivities_match_oracle(precision, gdtype, tol):
+    """Element and nodal sensitivities with full upstream gradients."""
+    phi, ref = oracle_16()
+    rng = np.random.default_rng(5)
+    dC, de, dk = rng.standard_normal((6, 6)), rng.standard_normal((3, 6)), rng.standard_normal((3, 3))
+    cell = make_cell(phi, precision=precision)
+    cell.solve()
+    P = ref["problem"]
+    g_rho = sensitivity.grad_rho(P, ref["y"], sensitivity.G_from_si(dC, de, dk, P.sc))
+    g_phi = ersatz.grad_phi(phi, g_rho)
+    for got, want in ((cell.sensitivity(dC, de, dk, dtype=gdtype), g_rho),
+                      (cell.sensitivity_phi(dC, de, dk, dtype=gdtype), g_phi)):
+        assert np.abs(got.double().cpu().numpy() - want).max() < tol * np.abs(want).max()
+
+
+@pytest.mark.parametrize("tc", [0, 1, 2])
+@pytest.mark.parametrize("n,axis", [(32, 0), (64, 2)])
+def test_laminate_closed_form(n, axis, tc):
+    from paper_2410_03148_gb300 import Cell
+    rho = cellgen.laminate_rho((n, n, n), axis, seed=7 + axis)
+    layers = {0: rho[0, 0, :], 1: rho[0, :, 0], 2: rho[:, 0, 0]}[axis]
+    cell = Cell(torch.as_tensor(np.ascontiguousarray(rho), device="cuda:0"), material(), kind="rho", tensor_cores=tc)
+    cell.solve()
+    assert close(cell.homogenise(), laminate.laminate_tensors(*material(), layers, axis)[:3], 1e-8)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_graphs_and_updates(precision):
+    """Direct launches, per-iteration graphs and the whole-solve graph, on a
+    fresh handle and on one that held another design, give the same bits."""
+    first, second = (cellgen.gaussian_levelset(16, seed=s) for s in (21, 22))
+    want = solved(second, precision=precision, graphs=0)
+    for graphs in (0, 1, 2):
+        c = make_cell(first, precision=precision, graphs=graphs)
+        c.solve()
+        c.update(torch.as_tensor(second, device="cuda:0"))
+        st = c.solve()
+        assert st["iters"] == want[0]["iters"] and st["rel_residual"] == want[0]["rel_residual"]
+        assert all(np.array_equal(x, y) for x, y in zip(c.homogenise(), want[1]))
+        c.close()
 
 
 @pytest.mark.parametrize("shape", [(24, 20, 32), (17, 16, 12)])
