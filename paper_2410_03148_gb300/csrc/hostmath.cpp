@@ -276,26 +276,41 @@ bool is_mm2(const double C[36], const double e[18], const double kap[9]) {
   return true;
 }
 
+namespace {
+// Unevaluated sum h + l with about 106 bits, in plain FP64 operations.
+struct Two {
+  double h, l;
+};
+Two two_sum(const Two& a, double bh, double bl) {
+  const double s = a.h + bh, t = s - a.h;
+  const double e = ((a.h - (s - t)) + (bh - t)) + (a.l + bl), h = s + e;
+  return {h, e - (h - s)};
+}
+}  // namespace
+
 void modal_matrix(const double* K, int nc, double* Km) {
   const int R = 8 * nc;
-  // 64 terms cancel: transformed in extended precision, so that the entries
-  // are the ones of K to its last digit
-  std::vector<long double> M(K, K + R * R);
-  for (int side = 0; side < 2; ++side)
+  // 64 terms cancel: transformed in pairs, so that the entries are the ones of
+  // K to its last digit.  (long double is software arithmetic on Arm, eight
+  // times slower, and has 64 bits on x86.)
+  std::vector<Two> M(R * R);
+  for (int i = 0; i < R * R; ++i) M[i] = {K[i], 0.0};
+  for (int side = 0; side < 2; ++side) {
+    const int along = side ? 1 : R, across = side ? R : 1;
     for (int bit = 1; bit < 8; bit <<= 1)
       for (int a = 0; a < 8; ++a) {
         if (a & bit) continue;
         for (int c = 0; c < nc; ++c)
           for (int k = 0; k < R; ++k) {
-            const int lo = a * nc + c, hi = (a | bit) * nc + c;
-            long double& u = side ? M[k * R + lo] : M[lo * R + k];
-            long double& v = side ? M[k * R + hi] : M[hi * R + k];
-            const long double s = v + u, d = v - u;   // sum at the clear bit, difference at the set one
+            Two& u = M[(a * nc + c) * along + k * across];
+            Two& v = M[((a | bit) * nc + c) * along + k * across];
+            const Two s = two_sum(v, u.h, u.l), d = two_sum(v, -u.h, -u.l);   // sum at the clear bit, difference at the set one
             u = s;
             v = d;
           }
       }
-  for (int i = 0; i < R * R; ++i) Km[i] = (double)(M[i] / 64.0L);
+  }
+  for (int i = 0; i < R * R; ++i) Km[i] = (M[i].h + M[i].l) / 64.0;
 }
 
 double child_weight(int c, int a, int B) {

@@ -3,7 +3,9 @@ called in the built library by their C++ names."""
 import ctypes
 import os
 import struct
+from fractions import Fraction
 
+import numpy as np
 import pytest
 
 LIB = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2410_03148_gb300", "libcell.so")
@@ -43,3 +45,23 @@ def test_gram_schmidt_chains_are_short(lib):
         b = blocks(length)
         assert 1 <= b <= 1024
         assert b >= min(1024, -(-length // (32 * 256))), n
+
+
+@pytest.mark.parametrize("nc", [1, 3, 4])
+def test_modal_matrix_is_the_rounded_exact_transform(lib, nc):
+    """H K H^T / 64 (H: sums and differences along the axes) of matrices whose
+    entries span 30 binary orders, against exact rational arithmetic: every
+    entry is the nearest double, whatever the host's long double is."""
+    fn = lib._ZN8cellhost12modal_matrixEPKdiPd
+    fn.argtypes, fn.restype = (ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p), None
+    R = 8 * nc
+    H = np.array([[np.prod([(1 if a >> b & 1 else -1) if m >> b & 1 else 1 for b in range(3)]) for a in range(8)] for m in range(8)])
+    for seed in range(12 // nc):
+        rng = np.random.default_rng(seed)
+        K = rng.uniform(-1, 1, (R, R)) * 2.0 ** -rng.integers(0, 30, (R, R))
+        got = np.empty((R, R))
+        fn(K.ctypes.data, nc, got.ctypes.data)
+        F = np.array([Fraction(v) for v in K.ravel()], dtype=object).reshape(8, nc, 8, nc)
+        want = np.einsum("ma,acbd->mcbd", H.astype(object), F)
+        want = np.einsum("nb,mcbd->mcnd", H.astype(object), want).reshape(R, R)
+        assert all(g == float(w / 64) for g, w in zip(got.ravel(), want.ravel()))
