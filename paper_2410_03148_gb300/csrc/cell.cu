@@ -376,6 +376,29 @@ void fill_modal(const double* Km, int nc, int o0, cell::ModalMat<V, NO, NI>& M, 
   }
 }
 
+// lambda_max(D^-1 K) of an element matrix in modal form, D = diag(K), kd[c] its
+// entry of component c.  D is the same at every corner and H / sqrt(8) is
+// orthogonal, so the spectrum is 8 times the one of the modal matrix scaled by
+// 1 / sqrt(kd), which splits into the groups of coupled modes (at most 4 dofs).
+double modal_lmax(const double* Km, const double* kd, int nc) {
+  const int R = 8 * nc;
+  double lmax = 0.0;
+  for (int c0 = 0; c0 < nc; ++c0)
+    for (int m0 = 1; m0 < 8; ++m0) {
+      int g[8], n = 0;
+      for (int d = 0; d < nc; ++d)
+        for (int m = 1; m < 8; ++m)
+          if (cell::modal_bits(m) == cell::modal_bits(m0) && cell::modal_couples(c0, m0, d, m)) g[n++] = m * nc + d;
+      if (g[0] != m0 * nc + c0) continue;   // the group's first dof stands for it
+      double A[64], lam[8], Q[64];
+      for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) A[i * n + j] = 8.0 * Km[g[i] * R + g[j]] / std::sqrt(kd[g[i] % nc] * kd[g[j] % nc]);
+      cellhost::sym_eig(A, n, lam, Q);
+      for (int i = 0; i < n; ++i) lmax = std::max(lmax, lam[i]);
+    }
+  return lmax;
+}
+
 template <typename T>
 void fill_modal_set(const double* Km, const double* Sm, ModalSet<T>& M) {
   auto conv = [](double v) { return (T)v; };
@@ -773,10 +796,14 @@ int alloc_mg_modal(cell_handle* h, BlockMG<T>& mg) {
     L.nz = n[2];
     L.nn = (i64)n[0] * n[1] * n[2];
     CKS(block_matrix(h, n, NC, L.kb));
-    L.lmax = cellhost::jacobi_lmax(L.kb.data(), R);
-    for (int c = 0; c < NC; ++c) L.dk[c] = (T)(1.0 / L.kb[c * R + c]);
+    double kd[NC];
+    for (int c = 0; c < NC; ++c) {
+      kd[c] = L.kb[c * R + c];
+      L.dk[c] = (T)(1.0 / kd[c]);
+    }
     std::vector<double> Km(R * R);
     cellhost::modal_matrix(L.kb.data(), NC, Km.data());
+    L.lmax = modal_lmax(Km.data(), kd, NC);
     if constexpr (NC == 3) fill_modal<3, 3, T>(Km.data(), 3, 0, L.uu, [](double v) { return (T)v; });
     else
       for (int m = 0; m < 8; ++m) L.ss.s[m] = (T)Km[m * 8 + m];
