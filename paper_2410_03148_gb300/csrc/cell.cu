@@ -1039,7 +1039,7 @@ void precond(cell_handle* h, const T* v, T* z, const int* mask) {
   if (h->modal) {
     cell::ModalArgs<T> m = modal_args<T>(h, z, len, K.tphi, nn, 9, mask);
     m.b = v + 3 * nn; m.bs = len;
-    cell::modal_pu<T>(m, modal_of<T>(h).pu, cell::MM_ADD, h->st);
+    cell::modal_pu<T>(m, modal_of<T>(h).pu, h->st);
   } else {
     cell::apply_pu<T>(a, K.K0, 9, h->st);
   }
@@ -1047,11 +1047,11 @@ void precond(cell_handle* h, const T* v, T* z, const int* mask) {
   block_solve<T, 1>(h, K.mgp, h->d.opt.vcycles_phi, K.tphi, nn, z + 3 * nn, len, K.rp, K.ep, mask);
 }
 
-// y = Ahat x, or y = b - Ahat x with b set.
+// y = Ahat x.
 template <typename T>
-void apply_full_T(cell_handle* h, const T* x, i64 xs, T* y, i64 ys, const T* b, i64 bs, const int* mask, int nrhs) {
+void apply_full_T(cell_handle* h, const T* x, i64 xs, T* y, i64 ys, const int* mask, int nrhs) {
   cell::ApplyArgs<T> a{};
-  a.x = x; a.xs = xs; a.y = y; a.ys = ys; a.b = b; a.bs = bs; a.alpha = b ? T(-1) : T(1); a.beta = T(1);
+  a.x = x; a.xs = xs; a.y = y; a.ys = ys; a.alpha = T(1);
   a.rho = rho_of<T>(h); a.nx = h->nx; a.ny = h->ny; a.nz = h->nz; a.active = mask;
   a.cslot1 = h->cslot1;
   const int pcls = sizeof(T) == 4 ? CELL_PROF_FULL32 : CELL_PROF_FULL64;
@@ -1064,15 +1064,30 @@ void apply_full_T(cell_handle* h, const T* x, i64 xs, T* y, i64 ys, const T* b, 
     }
   }
   if (!done && h->modal) {
-    cell::ModalArgs<T> m = modal_args<T>(h, x, xs, y, ys, nrhs, mask);
-    m.b = b; m.bs = bs;
-    cell::modal_full<T>(m, modal_of<T>(h).full, b ? cell::MM_RESID : cell::MM_APPLY, h->st);
+    cell::modal_full<T>(modal_args<T>(h, x, xs, y, ys, nrhs, mask), modal_of<T>(h).full, h->st);
   } else if (!done) {
     cell::FixedMat<T, 4> M;
     for (int i = 0; i < 1024; ++i) M.k[i] = (T)h->K0[i];
     cell::apply_full<T>(a, M, cell::AM_LINEAR, nrhs, h->st);
   }
   h->prof.end(pcls, ip, h->st);
+}
+
+// r64 = b64 - Ahat x64 of the masked loads in FP64 arithmetic (FP64 handles).
+void residual_f64(cell_handle* h, const int* mask) {
+  const i64 len = 4 * h->nn;
+  const int ip = h->prof.begin(h->st, CELL_PROF_FULL64);
+  if (h->modal) {
+    cell::ModalArgs<double> m = modal_args<double>(h, h->x64, len, h->r64, len, 9, mask);
+    m.b = h->b64; m.bs = len;
+    cell::modal_resid(m, h->m64.full, h->st);
+  } else {
+    cell::ApplyArgs<double> a{};
+    a.x = h->x64; a.xs = len; a.y = h->r64; a.ys = len; a.b = h->b64; a.bs = len; a.alpha = -1.0; a.beta = 1.0;
+    a.rho = h->rho64; a.nx = h->nx; a.ny = h->ny; a.nz = h->nz; a.active = mask;
+    cell::apply_full<double>(a, h->kd.K0, cell::AM_LINEAR, 9, h->st);
+  }
+  h->prof.end(CELL_PROF_FULL64, ip, h->st);
 }
 
 template <typename T>
@@ -1133,7 +1148,7 @@ void iteration(cell_handle* h, int j, cudaGraphConditionalHandle next = 0, bool 
   T* w = K.V + (i64)(j + 1) * vstride;
   T* zj = K.Z + (i64)j * vstride;
   precond<T>(h, vj, zj, h->active);
-  apply_full_T<T>(h, zj, len, w, len, nullptr, 0, h->active, 9);
+  apply_full_T<T>(h, zj, len, w, len, h->active, 9);
   const int ipk = h->prof.begin(s, CELL_PROF_KRYLOV);
   cell::GsArgs<T> a{};
   a.V = K.V; a.vstride = vstride; a.len = len;
@@ -1616,7 +1631,7 @@ int add_solve_graph(cell_handle* h, cudaGraph_t top) {
       if constexpr (sizeof(T) == 4)
         residual_df(h, h->b64, h->r64, 9, h->sel);
       else
-        apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, h->sel, 9);
+        residual_f64(h, h->sel);
       cell::dot<double>(h->r64, len, h->r64, len, len, h->partial, nblk, kNvMax, 9, nullptr, s);
       cell::reduce_partials(h->partial, nblk, 1, kNvMax, h->red, 0, 9, nullptr, s);
       cell::refine_ctl(h->bn2d, h->red, h->bfloor_d, P, h->want, h->tolabs, h->relres_d, h->iters_d, h->ctl_d, wh, s);
@@ -1779,7 +1794,7 @@ int solve_impl(cell_handle* h, cell_stats* st) {
       residual_df(h, h->b64, h->r64, 9, h->sel);
       h->prof.end(CELL_PROF_FULL64, ip, s);
     } else {
-      apply_full_T<double>(h, h->x64, len, h->r64, len, h->b64, len, h->sel, 9);
+      residual_f64(h, h->sel);
     }
   }
   // null-space projection (mean displacement and potential per load)
@@ -2317,9 +2332,9 @@ int cell_hilbert_velocity(cell_handle* h, double alpha, const double* dJ, const 
   for (int i = 0; i < ncons; ++i)
     if (!dC[i] || !std::isfinite(C[i])) return CELL_EINVAL;
   if (!std::isfinite(wJ) || !std::isfinite(wC)) return CELL_EINVAL;
-  // workspace: 2 (1 + ncons) nn doubles of the Krylov basis ((m + 1) x 9 x 4 nn values)
+  // workspace: 2 (1 + ncons) <= 18 nn doubles of the Krylov basis ((m + 1) x 9 x 4 nn
+  // values, m >= 1: at least 36 nn doubles)
   const bool mixed = h->d.opt.precision == CELL_MIXED_FP32;
-  if ((mixed ? (h->d.opt.restart + 1) / 2 : h->d.opt.restart + 1) < 1) return CELL_EINVAL;
   double* work = mixed ? reinterpret_cast<double*>(h->kf.V) : h->kd.V;
   const int st = cell::hilbert_velocity(h->nx, h->ny, h->nz, alpha, dJ, dC, C, ncons, wJ, wC, v, work, h->dptrs,
                                         h->partial, h->nblk, h->red, info, h->st);
@@ -2481,10 +2496,10 @@ int cell_apply(cell_handle* h, const void* x, void* y, int nrhs, int dtype) {
     if (h->modal) {
       if (dtype == CELL_F32)
         cell::modal_full<float>(modal_args<float>(h, static_cast<const float*>(x), len, static_cast<float*>(y), len,
-                                                  nrhs, nullptr), h->m32.full, cell::MM_APPLY, h->st);
+                                                  nrhs, nullptr), h->m32.full, h->st);
       else
         cell::modal_full<double>(modal_args<double>(h, static_cast<const double*>(x), len, static_cast<double*>(y),
-                                                    len, nrhs, nullptr), h->m64.full, cell::MM_APPLY, h->st);
+                                                    len, nrhs, nullptr), h->m64.full, h->st);
     } else if (dtype == CELL_F32) {
       cell::ApplyArgs<float> a{};
       a.x = static_cast<const float*>(x); a.xs = len; a.y = static_cast<float*>(y); a.ys = len;

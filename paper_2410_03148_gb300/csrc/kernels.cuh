@@ -196,8 +196,11 @@ struct ModalArgs {
   int nrhs;
   int rg;                  // loads per block, one after another (0 = 1)
 };
-template <typename T> void modal_full(const ModalArgs<T>& a, const ModalMat<T, 4, 4>& K, int mode, cudaStream_t s);
-template <typename T> void modal_pu(const ModalArgs<T>& a, const ModalMat<T, 1, 3>& K, int mode, cudaStream_t s);
+// y = Ahat x; y = b - Ahat x (FP64 only: the mixed solver's residual is
+// modal_resid_df); y = b + B x; any mode
+template <typename T> void modal_full(const ModalArgs<T>& a, const ModalMat<T, 4, 4>& K, cudaStream_t s);
+void modal_resid(const ModalArgs<double>& a, const ModalMat<double, 4, 4>& K, cudaStream_t s);
+template <typename T> void modal_pu(const ModalArgs<T>& a, const ModalMat<T, 1, 3>& K, cudaStream_t s);
 template <typename T> void modal_uu(const ModalArgs<T>& a, const ModalMat<T, 3, 3>& K, int mode, cudaStream_t s);
 template <typename T> void modal_ss(const ModalArgs<T>& a, const ModalSch<T>& K, int mode, cudaStream_t s);
 // FP64-grade r = b - Ahat x (r = Ahat x if b is null) in pairs of FP32, as resid_df

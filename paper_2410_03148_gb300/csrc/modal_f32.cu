@@ -18,7 +18,7 @@ int sm_count() {
 }  // namespace modal
 
 template <>
-void modal_full<float>(const ModalArgs<float>& a, const ModalMat<float, 4, 4>& K, int, cudaStream_t s) {
+void modal_full<float>(const ModalArgs<float>& a, const ModalMat<float, 4, 4>& K, cudaStream_t s) {
   modal::launch<MK_FULL, MM_APPLY, 3, 2, true, float>(a, K, s);
 }
 
@@ -34,7 +34,7 @@ void modal_full<float>(const ModalArgs<float>& a, const ModalMat<float, 4, 4>& K
 // 45 % of the instructions are not arithmetic (addresses, constant loads,
 // shuffles); the elastic step's bytes alone would take 150 us at 128^3.
 template <>
-void modal_pu<float>(const ModalArgs<float>& a, const ModalMat<float, 1, 3>& K, int, cudaStream_t s) {
+void modal_pu<float>(const ModalArgs<float>& a, const ModalMat<float, 1, 3>& K, cudaStream_t s) {
   modal::launch<MK_PU, MM_ADD, 4, 4, false, float>(a, K, s);
 }
 

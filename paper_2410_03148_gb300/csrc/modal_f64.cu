@@ -24,13 +24,15 @@ void go(const ModalArgs<double>& a, const K& k, cudaStream_t s) {
 }  // namespace
 
 template <>
-void modal_full<double>(const ModalArgs<double>& a, const ModalMat<double, 4, 4>& K, int mode, cudaStream_t s) {
-  if (mode == MM_APPLY) go<MK_FULL, MM_APPLY, 3, 2>(a, K, s);
-  else go<MK_FULL, MM_RESID, 3, 2>(a, K, s);
+void modal_full<double>(const ModalArgs<double>& a, const ModalMat<double, 4, 4>& K, cudaStream_t s) {
+  go<MK_FULL, MM_APPLY, 3, 2>(a, K, s);
+}
+void modal_resid(const ModalArgs<double>& a, const ModalMat<double, 4, 4>& K, cudaStream_t s) {
+  go<MK_FULL, MM_RESID, 3, 2>(a, K, s);
 }
 
 template <>
-void modal_pu<double>(const ModalArgs<double>& a, const ModalMat<double, 1, 3>& K, int, cudaStream_t s) {
+void modal_pu<double>(const ModalArgs<double>& a, const ModalMat<double, 1, 3>& K, cudaStream_t s) {
   go<MK_PU, MM_ADD, 4, 3>(a, K, s);
 }
 
