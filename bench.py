@@ -656,7 +656,7 @@ def main():
             "clocks": clocks,
             "detail": {"wall_s": wall, "step_ms": step_ms, "gmres_iters_max": iters,
                        "refinements": [s["refinements"] for s in stats],
-                       "tc_tiles_autotuned": {"elastic": stats[0]["tc_tiles"][0], "schur": stats[0]["tc_tiles"][1]},
+                       "coarse_loads_per_block": stats[0]["stencil_rg"],
                        "class_ms_per_step": share_ms, "class_share": class_share,
                        "class_source": "separate fully profiled pass over the first two designs "
                                        "(untimed); the timed region times only the roofline kernel"},

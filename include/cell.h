@@ -130,7 +130,9 @@ typedef struct cell_options {
                           the tensor-core smoothers' CTA tiles (x width 8/16/32 nodes, z-chunk
                           length) on this GPU and grid and keep the fastest per block (cell_stats
                           reports them); every tile gives bitwise the same result.  0 = widest
-                          tile and a wave-count heuristic.  MIXED (any tensor_cores): nonzero also
+                          tile and a wave-count heuristic.  (Solves of mm2 materials do not
+                          launch these kernels: there the tiles serve CELL_F32_TC block
+                          applies.)  MIXED (any tensor_cores): nonzero also
                           times the coarse levels' operator with 1, 3 and 9 loads per thread
                           (mm2 materials: per block, one after another) and keeps the fastest
                           per level (bitwise-neutral; cell_stats.stencil_rg). */
@@ -182,13 +184,15 @@ typedef struct cell_stats {
   int class_count[CELL_PROF_CLASSES];   /* profile: launches timed per class */
   long long class_units[CELL_PROF_CLASSES]; /* profile: sum over timed launches of the
                                            number of loads each launch processed */
-  int tc_tile_xt[2], tc_tile_L[2];  /* tensor-core smoother tile in use per block ([0] elastic
-                                       A, [1] Schur Sbar): x width in nodes and z-chunk length;
-                                       0 = not tuned (default tile or SIMT path) */
+  int tc_tile_xt[2], tc_tile_L[2];  /* tensor-core smoother tile per block ([0] elastic A, [1]
+                                       Schur Sbar; mm2 materials: of CELL_F32_TC block applies):
+                                       x width in nodes and z-chunk length; 0 = not tuned
+                                       (default tile or SIMT path) */
   double tc_tile_us[2];             /* the tuned tile's time per 9-load Chebyshev launch, us */
   int stencil_rg[2][8];             /* MIXED: loads per thread (mm2 materials: per block) of the
                                        coarse operator per multigrid level ([0] elastic, [1]
-                                       Schur; level 0 = fine grid, always 0); 0 = size default,
+                                       Schur; level 0 = fine grid, always 0; the first eight
+                                       levels of a deeper hierarchy); 0 = size default,
                                        1/3/9 = tuned at set-up (options.autotune; bitwise-neutral) */
 } cell_stats;
 
@@ -369,7 +373,8 @@ int cell_apply(cell_handle* h, const void* x, void* y, int nrhs, int dtype);
  * accumulation; any grid size).  Asynchronous on the handle's stream. */
 int cell_apply_block(cell_handle* h, int block, const void* x, void* y, int nrhs, int dtype);
 
-/* Set the CTA tile of the tensor-core smoother of one block (cell_block) for
+/* Set the CTA tile of the tensor-core smoother of one block (cell_block; for mm2
+ * materials it serves CELL_F32_TC block applies only) for
  * the rest of the handle's life, replacing the one cell_setup tuned or chose:
  * xt = nodes along x per CTA (8, 16 or 32, at most nx rounded up to a multiple
  * of 8), L = z-planes per CTA chunk (>= 1; values above nz act as nz); xt = L

@@ -1,12 +1,12 @@
 // Inverse of the coarsest multigrid level on the device (rediscretised
 // hierarchies): assembly from the element scales, FP32 Gauss-Jordan in the
 // registers of one block, two Newton-Schulz steps X <- X (2 I - A X) in FP64
-// over the whole chip.  On the host the FP64 factorisation of the default
-// coarsest level (192 unknowns) took 5 ms per design, half of an 8^3 design
-// step.  FP64 elimination in one block would take 1.7 ms (n^3 multiply-adds at
-// two per clock); the FP32 one takes 0.17 ms (0.9 us a pivot, bound by its
-// chain of barrier, shared-memory reads and update) and Newton-Schulz squares
-// its residual.
+// over the whole chip.  The FP64 factorisation of the default coarsest level
+// (192 unknowns) takes 5 ms per design on the host, more than an 8^3 design step.
+// FP64 elimination in one block would take 1.7 ms (n^3 multiply-adds at two per
+// clock); the FP32 one takes 0.17 ms (0.9 us a pivot, bound by its chain of
+// barrier, shared-memory reads and update) and Newton-Schulz (Schulz 1933)
+// squares its residual.
 #include "kernels.cuh"
 
 namespace cell {

@@ -9,11 +9,13 @@
 // sum c_i^2 |v_i|^2) and forms the dots of the new vector with the basis and
 // with itself: the Gram row of the next steps and the exact norm.  Basis
 // vectors are therefore normalised only approximately; their measured norms
-// nu_i enter every scalar.  Two basis passes and four launches per step; the
-// classical scheme with reorthogonalisation that this replaces took three
-// passes, a separate scaling and eleven launches (64^3: 310 us per step at 7
-// vectors, half of them FP64 additions of the block sums, which run at 1/64
-// rate; block sums are now pairs of FP32 with error-free additions).
+// nu_i enter every scalar.  (The low-synchronisation form of Swirydowicz, Langou,
+// Ananthan, Yang and Thomas, "Low synchronization Gram-Schmidt and generalized
+// minimal residual algorithms", 2021.)  Two basis passes and four launches per
+// step; classical Gram-Schmidt with selective reorthogonalisation takes three
+// passes, a scaling and eleven launches (64^3: 310 us per step at 7 vectors, half
+// of them FP64 additions of the block sums, which run at 1/64 rate).  Block sums
+// are pairs of FP32 with error-free additions.
 #include <algorithm>
 #include <cstdint>
 

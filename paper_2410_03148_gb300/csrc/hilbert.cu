@@ -278,8 +278,8 @@ int hilbert_velocity(int nx, int ny, int nz, double alpha, const double* dJ, con
   note_launch(), k_cheb_init<<<dim3(nb, nvec), kB, 0, s>>>(dptrs_dev, x, nn, 1.0 / theta);
   // The march pays its longer serial chain back from about 4e5 node values on
   // (us a step, node kernel against march: 96^3 x 4 200 / 151, 64^3 x 3 48 / 40,
-  // 48^3 x 3 24 / 26, 64^3 x 1 20 / 22, 30 x 33 x 27 x 2 7 / 17; before, with 27
-  // products and the direction form: 216, 53, 9);
+  // 48^3 x 3 24 / 26, 64^3 x 1 20 / 22, 30 x 33 x 27 x 2 7 / 17; 27 products a
+  // node and the direction form take 216, 53 and 9 where the better is 151, 40 and 7);
   // two blocks per SM, a chunk reads two planes more than it writes.
   const bool march = nn * nvec >= 400000;
   const i64 windows = ((i64)((ny + kRows - 1) / kRows) * (nx + 2) - 2 + kOut - 1) / kOut;

@@ -271,10 +271,10 @@ __global__ void k_elem_lmax(const T* __restrict__ ke, i64 ne, unsigned int* out)
   if (lam > 0.f) atomicMax(out, __float_as_uint(lam));
 }
 
-// x = Ainv b per load (nc comps of nn nodes, n = nc*nn).  A warp takes one row: its entries stay in registers (n <= 32 kRowRegs,
-// the rest is read again) and serve every load, lanes share the row and meet
-// in a shuffle sum.  (One thread per row chained n dependent loads: 7 to 15 us
-// at n = 192 against 3 us.)
+// x = Ainv b per load (nc comps of nn nodes, n = nc*nn).  A warp takes one row: its
+// entries stay in registers (n <= 32 kRowRegs, the rest is read again) and serve
+// every load, lanes share the row and meet in a shuffle sum: 3 us at n = 192 (one
+// thread per row chains n dependent loads, 7 to 15 us).
 constexpr int kRowRegs = 8;
 template <typename T>
 __global__ void __launch_bounds__(128)
