@@ -774,9 +774,20 @@ int block_matrix(const cell_handle* h, const int n[3], int nc, std::vector<doubl
       for (int b = 0; b < 8; ++b) M[a * 8 + b] = -K[(4 * a + 3) * 32 + 4 * b + 3];
     return CELL_OK;
   }
-  if (cellhost::local_schur(K, h->d.opt.schur_shift, S) != 0) {
-    set_error("elastic element block is not positive definite (check C)");
-    return CELL_EINVAL;
+  // the shift in proportion to the elastic block, as the finest grid's operator
+  // holds it (A_e grows with the element size); a shift at the rounding limit
+  // that the finest grid's factorisation bears may still fail here: raised then
+  double t0 = 0.0, tl = 0.0;
+  for (int i = 0; i < 32; ++i)
+    if (i % 4 != 3) t0 += h->K0[i * 33], tl += K[i * 33];
+  double shift = h->d.opt.schur_shift * (tl / t0);
+  int left = 32;
+  while (cellhost::local_schur(K, shift, S) != 0) {
+    if (--left == 0) {
+      set_error("elastic element block is not positive definite (check C)");
+      return CELL_EINVAL;
+    }
+    shift = std::max(4.0 * shift, 1e-18 * tl);
   }
   std::copy(S, S + 64, M.begin());
   return CELL_OK;
