@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(kBlock)
 k_resid_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs,
            const double* __restrict__ b, i64 bs, double* __restrict__ r, i64 rs,
            const float* __restrict__ rho_h, const float* __restrict__ rho_l,
-           const __grid_constant__ DFMat M, int nx, int ny, int nz, const int* active) {
+           const float* __restrict__ unscale, const __grid_constant__ DFMat M, int nx, int ny, int nz, const int* active) {
   const int q = blockIdx.z;
   if (active && !active[q]) return;
   NodeIdx t;
@@ -560,8 +560,9 @@ k_resid_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs,
       al[rp] = __ffma2_rn(sh[rp], wl2, __ffma2_rn(sl[rp], wh2, __fadd2_rn(al[rp], pe)));
     }
   }
-  const double v[4] = {(double)ah[0].x + (double)al[0].x, (double)ah[0].y + (double)al[0].y,
-                       (double)ah[1].x + (double)al[1].x, -((double)ah[1].y + (double)al[1].y)};
+  const float un = __ldg(unscale);   // the pair's scale, a power of two
+  const double v[4] = {(double)(ah[0].x * un) + (double)(al[0].x * un), (double)(ah[0].y * un) + (double)(al[0].y * un),
+                       (double)(ah[1].x * un) + (double)(al[1].x * un), -((double)(ah[1].y * un) + (double)(al[1].y * un))};
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const i64 o = (i64)c * t.nn + t.n;
@@ -732,13 +733,13 @@ void stencil_from_elem(const T* ke, T* st, int nx, int ny, int nz, cudaStream_t 
 }
 
 void resid_df(const float* xh, const float* xl, i64 xs, const double* b, i64 bs, double* r, i64 rs,
-              const float* rho_h, const float* rho_l, const DFMat& M, int nx, int ny, int nz,
+              const float* rho_h, const float* rho_l, const float* unscale, const DFMat& M, int nx, int ny, int nz,
               int nrhs, const int* active, cudaStream_t s) {
   ApplyArgs<float> a{};
   a.nx = nx;
   a.ny = ny;
   a.nz = nz;
-  note_launch(), k_resid_df<<<grid_for(a, nrhs), kBlock, 0, s>>>(xh, xl, xs, b, bs, r, rs, rho_h, rho_l, M,
+  note_launch(), k_resid_df<<<grid_for(a, nrhs), kBlock, 0, s>>>(xh, xl, xs, b, bs, r, rs, rho_h, rho_l, unscale, M,
                                                                   nx, ny, nz, active);
 }
 
@@ -756,6 +757,34 @@ void split_f64(const double* x, float* xh, float* xl, i64 n, cudaStream_t s) {
   i64 blocks = (n + 255) / 256;
   if (blocks > 8192) blocks = 8192;
   note_launch(), k_split<<<(unsigned)blocks, 256, 0, s>>>(x, xh, xl, n);
+}
+
+// Design scale of the double-float residual as an FP32 pair: rho_h + rho_l =
+// s rho with s a power of two that brings the root mean square (sumsq: device,
+// sum of rho^2) to about 1, *unscale = 1 / s.  Without it the low parts of the
+// products fall into FP32's subnormal range from rho of about 1e-25 down.
+// (Powers of two through the exponent bits: the library's frexp and division
+// cost more than the pass at 8^3.)
+__global__ void k_rho_pair(const double* __restrict__ rho, const double* __restrict__ sumsq, float* __restrict__ rho_h,
+                           float* __restrict__ rho_l, float* __restrict__ unscale, i64 n, double inv_n) {
+  // mean square = m 2^e with m in [1/2, 1); zero, infinite and NaN keep scale 1
+  const int bits = __double2hiint(__ldg(sumsq) * inv_n) >> 20;
+  int e = bits > 0 && bits < 2047 ? bits - 1022 : 0;
+  e = max(-120, min(120, e / 2));
+  const double s = __hiloint2double((1023 - e) << 20, 0);
+  for (i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (i64)gridDim.x * blockDim.x) {
+    const double v = rho[k] * s;
+    const float h = (float)v;
+    rho_h[k] = h;
+    rho_l[k] = (float)(v - (double)h);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *unscale = __int_as_float((127 + e) << 23);
+}
+
+void rho_pair(const double* rho, const double* sumsq, float* rho_h, float* rho_l, float* unscale, i64 n, cudaStream_t s) {
+  const i64 blocks = (n + 255) / 256;
+  note_launch(), k_rho_pair<<<(unsigned)(blocks < 8192 ? blocks : 8192), 256, 0, s>>>(rho, sumsq, rho_h, rho_l, unscale, n,
+                                                                                     1.0 / (double)n);
 }
 
 // ---- constant-bank slot manager ---------------------------------------------

@@ -272,8 +272,8 @@ struct cell_handle {
   double* drho = nullptr;   // level-set input: d rho_e / d phi_e (§2.6 smoothing)
   double* gtmp = nullptr;   // level-set input: element sensitivities before the chain
   double *b64 = nullptr, *x64 = nullptr, *r64 = nullptr;
-  // mixed path: x64 as FP32 pairs and rho's low part, for the double-float residual
-  float *xh = nullptr, *xl = nullptr, *rho_l = nullptr, *rho_tmp = nullptr;
+  // mixed path: x64 and rho as FP32 pairs (rho scaled), for the double-float residual
+  float *xh = nullptr, *xl = nullptr, *rho_h = nullptr, *rho_l = nullptr, *rho_unscale = nullptr;
   int* bad = nullptr;
   const double** dptrs = nullptr;   // device pointer table of cell_hilbert_velocity
   int* tc_err = nullptr;   // tensor-core kernels: expired bounded waits
@@ -1023,11 +1023,11 @@ cell::ModalArgs<T> modal_args(cell_handle* h, const T* x, i64 xs, T* y, i64 ys, 
 void residual_df(cell_handle* h, const double* b, double* r, int nrhs, const int* active) {
   const i64 len = 4 * h->nn;
   if (h->modal)
-    cell::modal_resid_df(h->xh, h->xl, len, b, len, r, len, h->rho32, h->rho_l, h->mdf, h->nx, h->ny, h->nz, nrhs,
-                         active, h->st);
+    cell::modal_resid_df(h->xh, h->xl, len, b, len, r, len, h->rho_h, h->rho_l, h->rho_unscale, h->mdf, h->nx, h->ny,
+                         h->nz, nrhs, active, h->st);
   else
-    cell::resid_df(h->xh, h->xl, len, b, len, r, len, h->rho32, h->rho_l, h->DF, h->nx, h->ny, h->nz, nrhs, active,
-                   h->st);
+    cell::resid_df(h->xh, h->xl, len, b, len, r, len, h->rho_h, h->rho_l, h->rho_unscale, h->DF, h->nx, h->ny, h->nz,
+                   nrhs, active, h->st);
 }
 
 // z = P_SCP^-1 v (§2.5.3): z_u ~ A^-1 v_u, z_phi ~ Sbar^-1 (v_phi + B z_u).
@@ -1300,9 +1300,8 @@ int load_design(cell_handle* h, const void* input) {
     else
       cell::rho_copy<double>(static_cast<const double*>(input), nn, h->rho32, h->rho64, h->bad, h->st);
   }
-  // rho_l = fp32(rho64 - rho32)
-  cell::split_f64(h->rho64, h->rho_tmp, h->rho_l, nn, h->st);
   cell::sum_reduce(h->rho64, nn, h->partial, h->nblk, h->red, h->st, 1);
+  cell::rho_pair(h->rho64, h->red, h->rho_h, h->rho_l, h->rho_unscale, nn, h->st);
   const bool mixed = d->opt.precision == CELL_MIXED_FP32;
   // mm2 materials: everything that follows is enqueued before the one wait
   if (h->modal) CKS(mixed ? fill_mg_modal<float>(h) : fill_mg_modal<double>(h));
@@ -1404,8 +1403,9 @@ int setup_impl(const cell_desc* d, cell_handle* h) {
     CKS(A.alloc(&h->drho, nn));
     CKS(A.alloc(&h->gtmp, nn));
   }
+  CKS(A.alloc(&h->rho_h, nn));
   CKS(A.alloc(&h->rho_l, nn));
-  CKS(A.alloc(&h->rho_tmp, nn));
+  CKS(A.alloc(&h->rho_unscale, 1));
   CKS(A.alloc(&h->bad, 1));
   CKS(A.alloc(&h->dense_dev, 2));
   CK(cudaMemsetAsync(h->dense_dev, 0, 2 * sizeof(unsigned), h->st));

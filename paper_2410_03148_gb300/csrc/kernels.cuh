@@ -205,8 +205,8 @@ template <typename T> void modal_uu(const ModalArgs<T>& a, const ModalMat<T, 3, 
 template <typename T> void modal_ss(const ModalArgs<T>& a, const ModalSch<T>& K, int mode, cudaStream_t s);
 // FP64-grade r = b - Ahat x (r = Ahat x if b is null) in pairs of FP32, as resid_df
 void modal_resid_df(const float* xh, const float* xl, i64 xs, const double* b, i64 bs, double* r, i64 rs,
-                    const float* rho_h, const float* rho_l, const ModalMat<DF, 4, 4>& K, int nx, int ny, int nz,
-                    int nrhs, const int* active, cudaStream_t s);
+                    const float* rho_h, const float* rho_l, const float* unscale, const ModalMat<DF, 4, 4>& K, int nx,
+                    int ny, int nz, int nrhs, const int* active, cudaStream_t s);
 
 // Constant-bank slots holding (K0, S0) in FP32 for the fixed-matrix kernels;
 // returns slot + 1, or 0 if none is free.  Release with cslot_release.
@@ -246,8 +246,11 @@ struct DFMat {
   float2 kl[512];
 };
 void resid_df(const float* xh, const float* xl, i64 xs, const double* b, i64 bs, double* r, i64 rs,
-              const float* rho_h, const float* rho_l, const DFMat& M, int nx, int ny, int nz,
+              const float* rho_h, const float* rho_l, const float* unscale, const DFMat& M, int nx, int ny, int nz,
               int nrhs, const int* active, cudaStream_t s);
+// rho as the scaled FP32 pair of the double-float residual: rho_h + rho_l = s rho, s a
+// power of two, *unscale = 1 / s; sumsq: device, sum of rho^2
+void rho_pair(const double* rho, const double* sumsq, float* rho_h, float* rho_l, float* unscale, i64 n, cudaStream_t s);
 // xh = fp32(x), xl = fp32(x - xh) for n values
 void split_f64(const double* x, float* xh, float* xl, i64 n, cudaStream_t s);
 // Tensor-core (tcgen05, 3xTF32) full-operator apply (apply_tc.cu); the grid

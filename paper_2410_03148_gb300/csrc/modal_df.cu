@@ -10,6 +10,7 @@ struct DfIO {
     double b[4];
   };
   const float *xh, *xl, *rh, *rl;
+  float un;   // 1 / scale of the rho pair (a power of two)
   const double* b;
   double* r;
   i64 nn;
@@ -26,7 +27,7 @@ struct DfIO {
   __device__ __forceinline__ void out(unsigned o, DF (&acc)[4], const DF (&)[4], const Pre& p) const {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      double v = (double)acc[c].h + (double)acc[c].l;
+      double v = (double)(acc[c].h * un) + (double)(acc[c].l * un);
       if (c == 3) v = -v;
       r[c * nn + o] = b ? p.b[c] - v : v;
     }
@@ -41,7 +42,7 @@ constexpr int kRows = 1, kBlocksPerSM = 2;
 __global__ void __launch_bounds__(modal::kThreads, kBlocksPerSM)
 k_modal_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs, const double* __restrict__ b, i64 bs,
            double* __restrict__ r, i64 rs, const float* __restrict__ rho_h, const float* __restrict__ rho_l,
-           const __grid_constant__ ModalMat<DF, 4, 4> K, int nx, int ny, int nz, const int* active, int L) {
+           const float* __restrict__ unscale, const __grid_constant__ ModalMat<DF, 4, 4> K, int nx, int ny, int nz, const int* active, int L) {
   const int q = blockIdx.y;
   if (active && !__any_sync(0xffffffffu, active[q])) return;
   DfIO io;
@@ -49,6 +50,7 @@ k_modal_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs, c
   io.xl = xl + q * xs;
   io.rh = rho_h;
   io.rl = rho_l;
+  io.un = __ldg(unscale);
   io.b = b ? b + q * bs : nullptr;
   io.r = r + q * rs;
   io.nn = (i64)nx * ny * nz;
@@ -59,11 +61,11 @@ k_modal_df(const float* __restrict__ xh, const float* __restrict__ xl, i64 xs, c
 }  // namespace
 
 void modal_resid_df(const float* xh, const float* xl, i64 xs, const double* b, i64 bs, double* r, i64 rs,
-                    const float* rho_h, const float* rho_l, const ModalMat<DF, 4, 4>& K, int nx, int ny, int nz,
-                    int nrhs, const int* active, cudaStream_t s) {
+                    const float* rho_h, const float* rho_l, const float* unscale, const ModalMat<DF, 4, 4>& K, int nx,
+                    int ny, int nz, int nrhs, const int* active, cudaStream_t s) {
   int L = 0;
   const dim3 grid = modal::grid_for(nx, ny, nz, nrhs, kRows, kBlocksPerSM, &L);
-  note_launch(), k_modal_df<<<grid, modal::kThreads, 0, s>>>(xh, xl, xs, b, bs, r, rs, rho_h, rho_l, K, nx, ny, nz, active, L);
+  note_launch(), k_modal_df<<<grid, modal::kThreads, 0, s>>>(xh, xl, xs, b, bs, r, rs, rho_h, rho_l, unscale, K, nx, ny, nz, active, L);
 }
 
 }  // namespace cell
